@@ -1388,6 +1388,31 @@ __device__ void negate_velocities(const Ctx& c, int n) {
 // ------------------------------------------------------------------------------------
 // FP64 end-point energies
 // ------------------------------------------------------------------------------------
+// The FP64 pipe of sm_103a takes 64 cycles per warp instruction (2 lanes per clock and SM),
+// so these sums are bound by their number of FP64 instructions alone.  The design keeps that
+// number low: a lane scans its row with integer arithmetic for the next pair to evaluate
+// (exact squared distance, cut-off test on it), so every FP64 instruction works on pairs
+// inside the cut-off; a pair belongs to the row of i < j when i + j is odd and of i > j
+// otherwise, which gives every row about half of its pairs (with j > i alone, the first
+// atoms own all of their pairs and the last ones none, and a warp waits for the fullest
+// row); 1/r comes from the FP32 rsqrt and one third-order step; erf(alpha r)/r from a table
+// of short polynomials whose small terms run in FP32; the terms of four pairs are added
+// by the multiply-adds that form them before one compensated addition.  Measured on 304
+// chains of 4000 ions at density 0.3: 2 ms per energy, against 41 ms for rows of j > i with
+// FP64 erfc, square root and divisions per pair; 152 aqueous chains of 9110 atoms: 13 ms
+// against 160 ms.  (ncu on the older form: FP64 pipe 78% busy, half of its lanes idle.)
+
+// float -> double of a positive normal value (exponent re-bias; exact)
+__device__ __forceinline__ double f2d_pos(float f) {
+  const unsigned b = __float_as_uint(f);
+  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+// float -> double, any sign (a zero becomes 2^-127)
+__device__ __forceinline__ double f2d(float f) {
+  const unsigned b = __float_as_uint(f);
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
 // U over atoms [0, n_tot) leaving out ex0/ex1/ex2 (-1 = none); each unordered pair once
 __device__ H4D_PHASE double energy64_impl(const Ctx& cref, int ex0, int ex1, int ex2);
 __device__ double energy64(const Ctx& c, int ex0, int ex1, int ex2 = -1) {
@@ -1396,6 +1421,35 @@ __device__ double energy64(const Ctx& c, int ex0, int ex1, int ex2 = -1) {
   if (c.tid == 0) c.R->t_energy_ns += (double)(gtimer() - t0);
   return u;
 }
+
+// part + the pair energy at r2 (LJ when lj, Coulomb when co), kqg = charge prefactor times
+// the screening
+__device__ __forceinline__ double pair_add64(const Pot& P, const CoulPiece* __restrict__ tab, int k, double r2, double kqg,
+                                             bool lj, bool co, double part) {
+  const float sf = (float)r2;
+  float y0;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(sf));
+  // r2 = 0 (two atoms on one grid point): 1/r is infinite, as r2 / r2 arithmetic has it
+  const double yd = sf > 1.2e-38f ? f2d_pos(y0) : __hiloint2double(0x7FF00000, 0);
+  // e = 1 - r2 y0^2 is below 4e-7: 1/r = y0 (1 + e/2 + 3/8 e^2), the next term below 2e-20
+  const double e = fma(-r2, yd * yd, 1.0);
+  const float ef = (float)e;
+  const double y = fma(f2d_pos(0.5f * y0), e + f2d_pos(0.75f * ef * ef), yd);
+  if (lj && __double2hiint(P.deps4[k]) != 0) {  // (tests on the high word: no FP64 compare)
+    const double y2 = y * y, y6 = y2 * y2 * y2;
+    part += fma(fma(P.dA12[k], y6, -P.dA6[k]), y6, -P.dljshift[k]);
+  }
+  if (co && (__double2hiint(kqg) << 1) != 0) {
+    const int m = min((int)(sf * P.etab_invw), P.etab_n - 1);
+    const CoulPiece c = tab[m];
+    const double h = r2 - c.sc;
+    const float hf = (float)h;
+    const float q = hf * fmaf(hf, fmaf(hf, c.c5, c.c4), c.c3);
+    part = fma(kqg, fma(h, fma(h, c.c2 + f2d(q), c.c1), c.c0) + y, part);
+  }
+  return part;
+}
+
 __device__ H4D_PHASE double energy64_impl(const Ctx& cref, int ex0, int ex1, int ex2) {
   const Ctx c = cref;
   const Eng& e = *c.e;
@@ -1403,41 +1457,72 @@ __device__ H4D_PHASE double energy64_impl(const Ctx& cref, int ex0, int ex1, int
   const Pot& P = e.pot;
   const GView& v = c.v;
   const int n = v.s->n_tot;
-  const double scale = R.L * 0x1.0p-32;
+  const double scale = R.L * 0x1.0p-32, scale2 = scale * scale;
   const double gscr = exp(-P.dkappa_sr * (double)v.s->w_cur);
-  const double rc2max = P.drc2_lj > P.drc2_c ? P.drc2_lj : P.drc2_c;
-  // per-atom Kahan sums over the row (j > i), then a sum over atoms in a fixed order;
-  // rows are taken by position k (atom ord[k])
+  // cut-offs on exact squared distances in fixed-point units
+  const u64 T_lj = (u64)ceil(P.drc2_lj / scale2), T_c = (u64)ceil(P.drc2_c / scale2);
+  const u64 T_max = T_lj > T_c ? T_lj : T_c;
+  // per-atom sums over the row, then a sum over atoms in a fixed order; rows are taken by
+  // position k (atom ord[k])
   const bool use_ord = v.s->n_ord == n;
-  for (int k = c.tid; k < n; k += c.T) {
-    const int i = use_ord ? (int)v.sorted[k] : k;
-    double acc = 0.0, comp = 0.0;
-    if (i == ex0 || i == ex1 || i == ex2) {
-      e.red[R.atom_off + i] = 0.0;
-      continue;
-    }
+  const int lane = c.tid & 31;
+  for (int k0 = c.tid - lane; k0 < n; k0 += c.T) {
+    const int k = k0 + lane;
+    const bool act = k < n;
+    const int i = act ? (use_ord ? (int)v.sorted[k] : k) : 0;
+    const bool own = act && i != ex0 && i != ex1 && i != ex2;
     const uint4 pi = v.pos[i];
     const int ti = type_of(i, R.nw3);
-    const double wi = (double)wbits(pi);
-    const int cnt = e.ncnt[R.atom_off + k];
-    for (int s = 0; s < cnt; ++s) {
-      const int j = e.nbr[nbr_index(e, R, k, s, c.ltpa)];
-      if (j <= i || j == ex0 || j == ex1 || j == ex2) continue;
-      const uint4 pj = v.pos[j];
-      const double dx = (double)(int)(pj.x - pi.x) * scale;
-      const double dy = (double)(int)(pj.y - pi.y) * scale;
-      const double dz = (double)(int)(pj.z - pi.z) * scale;
-      const double wj = (double)wbits(pj);
-      const double dw = wi - wj;
-      const double r2 = dx * dx + dy * dy + dz * dz + dw * dw;
-      if (r2 >= rc2max) continue;
-      const double g = ((wi != 0.0) != (wj != 0.0)) ? gscr : 1.0;
-      const double y = pair_u64(P, ti, type_of(j, R.nw3), r2, g) - comp;
-      const double t = acc + y;
-      comp = (t - acc) - y;
-      acc = t;
+    const float wi = wbits(pi);
+    const int cnt = own ? e.ncnt[R.atom_off + k] : 0;
+    double acc = 0.0, comp = 0.0, part = 0.0;
+    int s = 0, np = 0;
+    uint2 q = make_uint2(0u, 0u);
+    for (;;) {
+      bool have = false;
+      u64 d2 = 0;
+      int j = 0;
+      float wj = wi;
+      while (s < cnt && !have) {  // the row's next pair to evaluate
+        if ((s & 3) == 0) q = nbr_packets(e, R)[nbr_index(e, R, k, s, c.ltpa) / 4 - (size_t)R.atom_off * e.max_nbr / 4];
+        const unsigned half = (s & 2) ? q.y : q.x;
+        j = (int)((s & 1) ? half >> 16 : half & 0xFFFFu);
+        ++s;
+        if ((((i ^ j) & 1) ? i < j : i > j) && j != ex0 && j != ex1 && j != ex2) {
+          const uint4 pj = v.pos[j];
+          wj = wbits(pj);
+          d2 = fixed_d2(pi, pj);
+          have = d2 < T_max;
+        }
+      }
+      if (!__any_sync(0xffffffffu, have)) break;
+      if (have) {
+        const int tk = ti * 4 + type_of(j, R.nw3);
+        double r2 = __ull2double_rn(d2) * scale2;
+        double kqg = P.dkq[tk];
+        bool lj = d2 < T_lj, co = d2 < T_c;
+        if (wi != wj) {  // altitudes differ: one of the two flies
+          const double dw = (double)wi - (double)wj;
+          r2 = fma(dw, dw, r2);
+          lj = r2 < P.drc2_lj;
+          co = r2 < P.drc2_c;
+          if ((wi != 0.f) != (wj != 0.f)) kqg *= gscr;
+        }
+        if (P.etab_n > 0) {
+          part = pair_add64(P, e.etab, tk, r2, kqg, lj, co, part);
+        } else {
+          part += pair_u64(P, ti, tk - 4 * ti, r2, P.dkq[tk] != 0.0 ? kqg / P.dkq[tk] : 1.0);
+        }
+        if (++np == 4) {
+          const double y = part - comp, t = acc + y;
+          comp = (t - acc) - y;
+          acc = t;
+          part = 0.0;
+          np = 0;
+        }
+      }
     }
-    e.red[R.atom_off + i] = acc;
+    if (act) e.red[R.atom_off + i] = acc + (part - comp);
   }
   return fixed_order_sum(c, e.red + R.atom_off, n);
 }
