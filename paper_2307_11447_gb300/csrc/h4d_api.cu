@@ -315,12 +315,14 @@ static int coul_pieces(double alpha, double rc) {
   return std::max(1, (int)std::ceil(v / 0.0123));
 }
 
-static std::vector<CoulPiece> coul_table(const Pot& P, double alpha) {
-  std::vector<CoulPiece> t(std::max(P.etab_n, 1));
+static std::vector<CoulPiece> coul_table(double alpha, double rc) {
+  const int n = coul_pieces(alpha, rc);
+  const double shift = std::erfc(alpha * rc) / rc;
+  std::vector<CoulPiece> t(std::max(n, 1));
   std::memset(t.data(), 0, t.size() * sizeof(CoulPiece));
-  for (int k = 0; k < P.etab_n; ++k) {
+  for (int k = 0; k < n; ++k) {
     CoulPiece& c = t[k];
-    c.sc = (k + 0.5) * (P.drc2_c / P.etab_n);
+    c.sc = (k + 0.5) * (rc * rc / n);
     const double a2 = alpha * alpha, v = a2 * c.sc, ev = std::exp(-v);
     double I[7], term = 1.0, sum = 0.0;
     for (int q = 1; q < 200 && term > 1e-18 * sum; ++q) {
@@ -334,7 +336,7 @@ static std::vector<CoulPiece> coul_table(const Pot& P, double alpha) {
     double f = -alpha * kC, cm[6];
     const double f_lo = std::fma(-alpha, kC, -f) - alpha * kClo;
     for (int m = 0; m < 6; ++m) {
-      cm[m] = m == 0 ? std::fma(f, I[0], f_lo * I[0] - P.dshift_c) : f * I[m];
+      cm[m] = m == 0 ? std::fma(f, I[0], f_lo * I[0] - shift) : f * I[m];
       f *= -a2 / (m + 1);
     }
     c.c0 = cm[0];
@@ -522,10 +524,7 @@ static int alloc_all(h4d_ctx* c) {
   CK(cudaMalloc(&c->d_lord, na * sizeof(uint16_t)));
   CK(cudaMalloc(&c->d_red, na * sizeof(double)));
   {
-    Pot P;
-    Proto pr;
-    fill_pot(c->prm, P, pr);
-    const std::vector<CoulPiece> tab = coul_table(P, c->prm.alpha);
+    const std::vector<CoulPiece> tab = coul_table(c->prm.alpha, c->prm.rc_coul);
     CK(cudaMalloc(&c->d_etab, tab.size() * sizeof(CoulPiece)));
     CK(cudaMemcpy(c->d_etab, tab.data(), tab.size() * sizeof(CoulPiece), cudaMemcpyHostToDevice));
   }
@@ -1688,7 +1687,7 @@ extern "C" int h4d_eval_forces_static(const h4d_params* params, double L, int32_
   const size_t o_red = carve_bytes(off, na * sizeof(double));
   std::memset(&c.eng, 0, sizeof(Eng));
   fill_pot(c.prm, c.eng.pot, c.eng.proto);
-  const std::vector<CoulPiece> etab = coul_table(c.eng.pot, c.prm.alpha);
+  const std::vector<CoulPiece> etab = coul_table(c.prm.alpha, c.prm.rc_coul);
   const size_t o_tab = carve_bytes(off, etab.size() * sizeof(CoulPiece));
   if (off > kStaticScratchBytes) return H4D_ECAPACITY;  // too many atoms for 16 MiB
 

@@ -322,9 +322,9 @@ __device__ __forceinline__ GView carve(char* base, int cap_atoms, int nc, int nt
   return v;
 }
 
-// The sentinel slot after a replica's last possible atom: row padding (kNoAtom) is read
-// as min(index, cap_atoms), i.e. as this slot, whose infinite altitude puts it beyond every
-// cut-off, so padding needs neither a branch nor a mask in the pair loop.
+// The sentinel slot after a replica's last possible atom: Verlet rows are padded with its
+// index (cap_atoms); its infinite altitude puts it beyond every cut-off, so padding needs
+// neither a branch nor a mask in the pair loop.
 __device__ __forceinline__ void write_sentinel(const GView& v, int cap_atoms) {
   v.pos[cap_atoms] = make_uint4(0u, 0u, 0u, 0x7F800000u);
 }
@@ -381,10 +381,7 @@ __device__ __forceinline__ size_t packet_index(const Eng& e, const RepC& R, int 
 __device__ __forceinline__ size_t nbr_index(const Eng& e, const RepC& R, int i, int s, int ltpa) {
   return packet_index(e, R, i, s >> 2, ltpa) * 4 + (s & 3);
 }
-// outer rows: one lane per atom (packets of four indices, consecutive atoms adjacent)
-__device__ __forceinline__ size_t out_packet_index(const Eng& e, const RepC& R, int i, int P) {
-  return (size_t)R.atom_off * e.max_out / 4 + (size_t)P * R.cap_atoms + i;
-}
+// outer rows: slot s of the row at position k is element s%4 of packet (s/4) cap_atoms + k
 __device__ __forceinline__ const uint2* out_packets(const Eng& e, const RepC& R) {
   return reinterpret_cast<const uint2*>(e.nbr_out + (size_t)R.atom_off * e.max_out);
 }
@@ -463,29 +460,6 @@ __device__ __forceinline__ u64 gtimer() {
   return t;
 }
 
-// four row entries collected in a 64-bit shift register and stored as one 8-byte packet
-// (first entry in the low 16 bits); a partial packet is completed with kNoAtom
-struct RowBuf {
-  unsigned long long b;
-  int n;
-  __device__ __forceinline__ void init() { b = ~0ull; n = 0; }
-  __device__ __forceinline__ void put(int j) {
-    b = (b >> 16) | ((unsigned long long)(unsigned)j << 48);
-    ++n;
-  }
-  // put(j) when ok, with selects instead of a branch
-  __device__ __forceinline__ void put_if(bool ok, int j) {
-    const unsigned long long nb = (b >> 16) | ((unsigned long long)(unsigned)j << 48);
-    b = ok ? nb : b;
-    n += ok ? 1 : 0;
-  }
-  __device__ __forceinline__ uint2 packet() const {
-    const unsigned long long x = b >> (16 * (4 - n));  // shift in kNoAtom for missing entries
-    const unsigned long long y = x | (n == 4 ? 0ull : (~0ull << (16 * n)));
-    return make_uint2((unsigned)y, (unsigned)(y >> 32));
-  }
-};
-
 // ------------------------------------------------------------------------------------
 // Neighbour list: fixed-point cells, deterministic stable counting sort, full rows
 // ------------------------------------------------------------------------------------
@@ -546,6 +520,156 @@ __device__ void refresh_list(const Ctx& c) {
     c.R->refreshes++;
   }
 }
+// Entries of a lane's row collected in a register pair, first entry lowest: an accepted
+// 16-bit index is shifted in by byte permutes and a full pair is one packet store, all
+// predicated.  The row's packets are cap_atoms apart (outer rows and Verlet rows of one lane)
+// or, with tpa lanes per Verlet row (T1 false), dealt as packet_index does.
+template <bool T1>
+struct RowOut {
+  uint2* base;    // first packet of the replica
+  unsigned wo;    // offset of the next packet
+  unsigned cap, tpa;
+  int cnt, max;   // entries so far, capacity (a multiple of 4)
+  unsigned lo, hi;
+  __device__ __forceinline__ RowOut(uint2* b, unsigned pos, unsigned cap_, unsigned tpa_, int ltpa, int max_)
+      : base(b), wo(pos << (T1 ? 0 : ltpa)), cap(cap_), tpa(tpa_), cnt(0), max(max_), lo(0u), hi(0u) {}
+  // the entry is the low (sel 0x5432) or the high (0x7632) half of word
+  __device__ __forceinline__ void put(bool ok, unsigned word, unsigned sel) {
+    lo = ok ? __byte_perm(lo, hi, 0x5432) : lo;
+    hi = ok ? __byte_perm(hi, word, sel) : hi;
+    cnt += ok ? 1 : 0;
+    if (ok && (cnt & 3) == 0 && cnt <= max) {
+      base[wo] = make_uint2(lo, hi);
+      if (T1) wo += cap;
+      else wo += (((unsigned)cnt >> 2) & (tpa - 1)) ? 1u : cap * tpa - (tpa - 1);
+    }
+  }
+  // the last partial packet, completed with pad2 (two entries); true when the row overflowed
+  // (cnt is then cut to whole packets)
+  __device__ __forceinline__ bool finish(unsigned pad2) {
+    const int r = cnt & 3;
+    if (r > 0 && cnt <= max) {  // the r entries are at the top of (lo, hi)
+      uint2 t;
+      t.x = r == 1 ? __byte_perm(hi, pad2, 0x5432) : (r == 2 ? hi : __byte_perm(lo, hi, 0x5432));
+      t.y = r == 3 ? __byte_perm(hi, pad2, 0x5432) : pad2;
+      base[wo] = t;
+    }
+    if (cnt <= max) return false;
+    cnt = max & ~3;
+    return true;
+  }
+};
+
+// Outer rows.  A warp takes up to 32 home atoms of a cell, one per lane, and streams the
+// candidates of the 27 stencil cells past them (every lane reads the same shared-memory word).
+// Test and append are separate: the test of a candidate is three instructions (byte-wise
+// difference, dot product with itself minus the threshold, sign bit shifted into a 32-bit
+// mask), and each lane then takes only its accepted candidates out of the mask.  Bound: the
+// half-rate ALU pipe.  An outer build and its filter for 304 chains of 4000 ions: 4.2 -> 3.0
+// ms (152 aqueous chains: 21.6 -> 12.1 ms); testing and appending in one step per candidate took 35 instructions, and a ballot
+// compaction with one candidate per lane was held up by its popcounts (8 cycles each).
+// Cells are visited in a fixed order and hold their atoms in ascending index order, and z
+// neighbours are one run of the sorted list, so a row does not depend on the thread mapping.
+// Work items (cell, home pass) are handed out through a shared counter, so clustered (dense)
+// cells do not leave one warp with all the work.  Without cells (small boxes) item k is the
+// k-th chunk of 32 atoms and every atom is a candidate, in index order.  Returns whether a row
+// overflowed.
+template <bool CELLS, bool WATER>
+__device__ __forceinline__ int outer_rows(const Ctx& c, int n, bool use_rank) {
+  const Eng& e = *c.e;
+  const RepC& R = c.r;
+  const GView& v = c.v;
+  const int nc = R.nc, lane = c.tid & 31;
+  const int n_items = CELLS ? v.s->n_items : (n + 31) >> 5;
+  uint2* rows = reinterpret_cast<uint2*>(e.nbr_out) + (size_t)R.atom_off * e.max_out / 4;
+  int overflow = 0;
+  for (;;) {
+    int item = 0;
+    if (lane == 0) item = atomicAdd(&v.s->next_item, 1);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item >= n_items) break;
+    int cell = 0, h0 = 32 * item, h1 = min(h0 + 32, n);
+    if (CELLS) {  // last cell whose first item is <= item (binary search on the prefix)
+      int a = 0, b = nc * nc * nc - 1;
+      while (a < b) {
+        const int mid = (a + b + 1) >> 1;
+        if (v.cfill[mid] <= item) a = mid; else b = mid - 1;
+      }
+      cell = a;
+      h0 = v.cstart[cell] + 32 * (item - v.cfill[cell]);
+      h1 = min(h0 + 32, v.cstart[cell + 1]);
+    }
+    const int hq = h0 + lane;
+    const int ih = hq < h1 ? (CELLS ? (int)v.sorted[hq] : hq) : (int)kNoAtom;
+    const bool act = ih != (int)kNoAtom;
+    const int i = act ? ih : 0;
+    const unsigned pos = use_rank ? (unsigned)e.lrank[R.atom_off + i] : (unsigned)i;  // where this atom's rows go
+    const uint4 pi = v.pos[i];
+    // left out: the atom itself or, for a water's atom, its molecule
+    const unsigned ex0 = WATER && i < R.nw3 ? (unsigned)(i - i % 3) : (unsigned)i;
+    const unsigned exn = WATER && i < R.nw3 ? 3u : 1u;
+    RowOut<true> row(rows, pos, (unsigned)R.cap_atoms, 1u, 0, e.max_out);
+    // accepted candidates: bit 31 of m is the first of the candidates from q0 on
+    auto take = [&](unsigned m, int q0) {
+      while (m) {
+        const int z = __clz((int)m);
+        m &= ~(0x80000000u >> z);
+        const int j = CELLS ? (int)v.sorted[q0 + z] : q0 + z;
+        row.put(j != (int)kNoAtom && (unsigned)j - ex0 >= exn, (unsigned)j, 0x5432);
+      }
+    };
+    if (CELLS) {
+      const unsigned pi8 = pack8(pi);
+      // conservative test at 8-bit resolution (the Verlet filter applies the exact criterion).
+      // The byte of |a - b|, read as a signed byte, is the minimum-image difference up to sign.
+      const int thr = act ? -(int)R.T8_out - 1 : 0;
+      const int cx = cell / (nc * nc), cy = (cell / nc) % nc, cz = cell % nc;
+      for (int d = 0; d < 9; ++d) {
+        int ex = cx + d / 3 - 1, ey = cy + d % 3 - 1;
+        ex += (ex < 0) ? nc : 0; ex -= (ex >= nc) ? nc : 0;
+        ey += (ey < 0) ? nc : 0; ey -= (ey >= nc) ? nc : 0;
+        const int col = (ex * nc + ey) * nc;
+        // z - 1, z, z + 1 in order: one run of the sorted list, two where the box wraps
+        for (int w = 0; w < 2; ++w) {
+          int z0, z1;
+          if (cz == 0) { z0 = w == 0 ? nc - 1 : 0; z1 = w == 0 ? nc - 1 : 1; }
+          else if (cz == nc - 1) { z0 = w == 0 ? nc - 2 : 0; z1 = w == 0 ? nc - 1 : 0; }
+          else { if (w) break; z0 = cz - 1; z1 = cz + 1; }
+          const int s0 = v.cstart[col + z0], s1 = v.cstart[col + z1 + 1];
+          for (int q0 = s0; q0 < s1; q0 += 32) {
+            const int len = min(32, s1 - q0);  // a multiple of 4
+            unsigned m = 0u;
+            for (int q = 0; q < len; q += 4) {
+              const uint4 c8 = *reinterpret_cast<const uint4*>(v.sorted8 + q0 + q);
+              const unsigned cu[4] = {c8.x, c8.y, c8.z, c8.w};
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const int t = (int)__vabsdiffu4(pi8, cu[u]);
+                m = __funnelshift_l((unsigned)__dp4a(t, t, thr), m, 1);
+              }
+            }
+            take(m << (32 - len), q0);
+          }
+        }
+      }
+    } else {
+      for (int q0 = 0; q0 < n; q0 += 32) {
+        const int len = min(32, n - q0);
+        unsigned m = 0u;
+        for (int q = 0; q < len; ++q) m = 2u * m + (act && d2_16(pi, v.pos[q0 + q]) <= R.T16_out ? 1u : 0u);
+        take(m << (32 - len), q0);
+      }
+    }
+    if (act) {
+      if (row.finish(0u)) overflow = 1;
+      e.ncnt_out[R.atom_off + pos] = row.cnt;
+      e.ref_out[R.atom_off + i] = pi;
+      if (use_rank) e.lord[R.atom_off + pos] = (uint16_t)i;
+    }
+  }
+  return overflow;
+}
+
 // Each phase of the engine is a function of its own (not inlined), with the context copied
 // to locals at entry: its loops get the whole register budget instead of sharing it with
 // whatever the caller keeps live across the call.
@@ -614,124 +738,15 @@ __device__ H4D_PHASE void build_list_impl(const Ctx& cref) {
         if (k < ncell) v.cfill[k] = carry2 + incl - x;
         carry2 += __shfl_sync(0xffffffffu, incl, 31);
       }
-      if (lane == 0) { v.s->n_items = carry2; v.s->next_item = 0; }
+      if (lane == 0) v.s->n_items = carry2;
     }
     c.sync();
   }
-  // Rows: one warp per cell, its lanes holding up to 32 home atoms of the cell at a time.
-  // The candidates of the 27 stencil cells stream through the warp one at a time, so
-  // every lane reads the same shared-memory word (broadcast, no bank conflicts); each lane
-  // appends the accepted candidates to its own row.  Cells are visited in a fixed order
-  // and hold their atoms in ascending index order, so a row does not depend on the thread
-  // mapping.  Without cells (small boxes) every atom is a candidate of every atom.
-  const int nwarps = c.T >> 5, warp = c.tid >> 5, lane = c.tid & 31;
-  // without cells, "cell" k is the k-th chunk of 32 home atoms and every atom is a candidate
-  const int ncell_rows = (nc > 0) ? nc * nc * nc : (n + 31) / 32;
-  const int maxo = e.max_out;
-  const bool has_water = R.nw3 > 0;  // uniform: the exclusion test only where waters exist
-  int overflow = 0;
-  // Work items are (cell, home pass of up to 32 atoms), handed out through a shared
-  // counter so clustered (dense) cells do not leave one warp with all the work.  Without
-  // cells, item k is the k-th chunk of 32 home atoms, assigned round-robin.
-  for (int it = 0;; ++it) {
-    int item;
-    if (nc > 0) {
-      if (lane == 0) item = atomicAdd(&v.s->next_item, 1);
-      item = __shfl_sync(0xffffffffu, item, 0);
-      if (item >= v.s->n_items) break;
-    } else {
-      item = warp + it * nwarps;
-      if (item >= ncell_rows) break;
-    }
-    int cell = 0, pass = item;
-    if (nc > 0) {  // last cell whose first item is <= item (binary search on the prefix)
-      int lo = 0, hi = ncell_rows - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (v.cfill[mid] <= item) lo = mid; else hi = mid - 1;
-      }
-      cell = lo;
-      pass = item - v.cfill[lo];
-    }
-    const int h0 = (nc > 0) ? v.cstart[cell] + 32 * pass : 32 * item;
-    const int h1 = (nc > 0) ? min(h0 + 32, v.cstart[cell + 1]) : min(32 * item + 32, n);
-    if (nc == 0) cell = 0;
-    const int cx = (nc > 0) ? cell / (nc * nc) : 0;
-    const int cy = (nc > 0) ? (cell / nc) % nc : 0;
-    const int cz = (nc > 0) ? cell % nc : 0;
-    for (int hb = h0; hb < h1; hb += 32) {
-      const int hq = hb + lane;
-      const int ih = (hq < h1) ? ((nc > 0) ? (int)v.sorted[hq] : hq) : (int)kNoAtom;
-      const bool act = ih != (int)kNoAtom;
-      const int i = act ? ih : 0;
-      const int pos = use_rank ? (int)e.lrank[R.atom_off + i] : i;  // where this atom's rows go
-      const uint4 pi = v.pos[i];
-      const unsigned pi8 = pack8(pi);
-      int cnt = 0;
-      RowBuf rb;
-      rb.init();
-      const int nst = (nc > 0) ? 27 : 1;
-      for (int d = 0; d < nst; ++d) {
-        int s0 = 0, s1 = n;
-        if (nc > 0) {
-          int ex = cx + d / 9 - 1, ey = cy + (d / 3) % 3 - 1, ez = cz + d % 3 - 1;
-          ex += (ex < 0) ? nc : 0; ex -= (ex >= nc) ? nc : 0;
-          ey += (ey < 0) ? nc : 0; ey -= (ey >= nc) ? nc : 0;
-          ez += (ez < 0) ? nc : 0; ez -= (ez >= nc) ? nc : 0;
-          const int cc = (ex * nc + ey) * nc + ez;
-          s0 = v.cstart[cc];
-          s1 = v.cstart[cc + 1];
-        }
-        // Four candidates per iteration.  With cells: one 8-byte index load and one 16-byte
-        // load of their packed 8-bit coordinates; the per-byte wrapping difference is the
-        // minimum image at 8-bit resolution and __dp4a squares it (a conservative test:
-        // the Verlet filter applies the exact criterion).  Without cells: 16-bit test.
-        for (int q = s0; q < s1; q += 4) {
-          int jj[4];
-          bool near[4];
-          if (nc > 0) {
-            const uint2 w4 = *reinterpret_cast<const uint2*>(v.sorted + q);
-            const uint4 c8 = *reinterpret_cast<const uint4*>(v.sorted8 + q);
-            jj[0] = (int)(w4.x & 0xFFFFu); jj[1] = (int)(w4.x >> 16);
-            jj[2] = (int)(w4.y & 0xFFFFu); jj[3] = (int)(w4.y >> 16);
-            const unsigned cu[4] = {c8.x, c8.y, c8.z, c8.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int d = (int)__vsub4(pi8, cu[u]);
-              near[u] = __dp4a(d, d, 0) <= (int)R.T8_out;
-            }
-          } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              jj[u] = (q + u < s1) ? q + u : (int)kNoAtom;
-              near[u] = d2_16(pi, v.pos[jj[u] == kNoAtom ? i : jj[u]]) <= R.T16_out;
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int j = jj[u];
-            const bool ok = act && near[u] && (j != (int)kNoAtom) && (j != i) &&
-                            !(has_water && excluded_pair(i, j, R.nw3));
-            rb.put_if(ok, j);
-            cnt += ok ? 1 : 0;
-            if (rb.n == 4) {
-              if (cnt <= maxo)
-                reinterpret_cast<uint2*>(e.nbr_out)[out_packet_index(e, R, pos, (cnt - 1) >> 2)] = rb.packet();
-              rb.init();
-            }
-          }
-        }
-      }
-      if (act) {
-        if (rb.n > 0 && cnt <= maxo)  // last partial packet, padded with kNoAtom
-          reinterpret_cast<uint2*>(e.nbr_out)[out_packet_index(e, R, pos, (cnt - 1) >> 2)] = rb.packet();
-        if (cnt > maxo) { overflow = 1; cnt = maxo & ~3; }
-        e.ncnt_out[R.atom_off + pos] = cnt;
-        e.ref_out[R.atom_off + i] = pi;
-        if (use_rank) e.lord[R.atom_off + pos] = (uint16_t)i;
-      }
-    }
-  }
+  if (c.tid == 0) v.s->next_item = 0;
+  c.sync();
+  int overflow;
+  if (nc == 0) overflow = R.nw3 > 0 ? outer_rows<false, true>(c, n, use_rank) : outer_rows<false, false>(c, n, use_rank);
+  else overflow = R.nw3 > 0 ? outer_rows<true, true>(c, n, use_rank) : outer_rows<true, false>(c, n, use_rank);
   if (overflow) atomicOr(&v.s->flag_overflow, 1);
   c.sync();
   if (c.tid == 0) {
@@ -788,6 +803,52 @@ __device__ void next_rank(const Ctx& c, int n, bool lay) {
   c.sync();
 }
 
+// One lane per row: four candidates per packet, the exact test, and the predicated append of
+// RowOut (appending through 64-bit shifts and selects with a branch at each full packet took a
+// third longer).  The last Verlet packet is padded with the sentinel's index.  Bound:
+// shared-memory position gathers and the ALU pipe.  Returns whether a row overflowed.
+template <bool T1>
+__device__ __forceinline__ int filter_rows(const Ctx& c, int n, bool lay) {
+  const Eng& e = *c.e;
+  const RepC& R = c.r;
+  const GView& v = c.v;
+  const int maxn = e.max_nbr;
+  const uint2* pko = out_packets(e, R);
+  const unsigned cap = (unsigned)R.cap_atoms;
+  uint2* nbr2 = reinterpret_cast<uint2*>(e.nbr) + (size_t)R.atom_off * maxn / 4;
+  const u64 T_list = R.T_list;
+  int overflow = 0;
+  for (int k = c.tid; k < n; k += c.T) {
+    const int i = lay ? (int)e.lord[R.atom_off + k] : k;
+    if (lay) v.sorted[k] = (uint16_t)i;
+    const uint4 pi = v.pos[i];
+    const int cnt_out = e.ncnt_out[R.atom_off + k];
+    const int npk = (cnt_out + 3) >> 2;
+    RowOut<T1> row(nbr2, (unsigned)k, cap, (unsigned)c.tpa, c.ltpa, maxn);
+    const uint2* src = pko + k;
+    uint2 q = (npk > 0) ? src[0] : make_uint2(0u, 0u);
+    for (int p = 0; p < npk; ++p) {
+      const uint2 qn = (p + 1 < npk) ? src[(size_t)(p + 1) * cap] : make_uint2(0u, 0u);
+      if (H4D_PF_FILTER > 0 && p + H4D_PF_FILTER < npk) prefetch_l2(src + (size_t)(p + H4D_PF_FILTER) * cap);
+      const int left = cnt_out - 4 * p;  // entries of this packet; the others are not read
+      const int j0 = (int)(q.x & 0xFFFFu);
+      const int j1 = left > 1 ? (int)(q.x >> 16) : i;
+      const int j2 = left > 2 ? (int)(q.y & 0xFFFFu) : i;
+      const int j3 = left > 3 ? (int)(q.y >> 16) : i;
+      const uint4 p0 = v.pos[j0], p1 = v.pos[j1], p2 = v.pos[j2], p3 = v.pos[j3];
+      row.put(fixed_d2(pi, p0) <= T_list, q.x, 0x5432);
+      row.put(left > 1 && fixed_d2(pi, p1) <= T_list, q.x, 0x7632);
+      row.put(left > 2 && fixed_d2(pi, p2) <= T_list, q.y, 0x5432);
+      row.put(left > 3 && fixed_d2(pi, p3) <= T_list, q.y, 0x7632);
+      q = qn;
+    }
+    if (row.finish(cap | (cap << 16))) overflow = 1;
+    e.ncnt[R.atom_off + k] = row.cnt;
+    e.ref[R.atom_off + i] = pi;
+  }
+  return overflow;
+}
+
 // Verlet rows filtered from the outer rows: one thread per atom streams its outer row
 // (one 8-byte packet load per four candidates) and keeps the candidates inside r_list, in
 // outer-row order, so the Verlet rows are as deterministic as the outer ones.
@@ -797,50 +858,10 @@ __device__ H4D_PHASE void filter_list_impl(const Ctx& cref) {
   const RepC& R = c.r;
   const GView& v = c.v;
   const int n = v.s->n_tot;
-  const int ltpa = c.ltpa;
-  const int maxn = e.max_nbr;
-  const uint2* pko = out_packets(e, R);
-  const size_t ostride = (size_t)R.cap_atoms;
-  int overflow = 0;
   // positions k of the outer rows' layout (atom lord[k], or k when rows are by index): the
   // outer rows are read and the Verlet rows written at the same position, both coalesced
   const bool lay = v.s->n_lay == n;
-  for (int k = c.tid; k < n; k += c.T) {
-    const int i = lay ? (int)e.lord[R.atom_off + k] : k;
-    if (lay) v.sorted[k] = (uint16_t)i;
-    const int pos = k;
-    const uint4 pi = v.pos[i];
-    const int cnt_out = e.ncnt_out[R.atom_off + pos];
-    const int npk = (cnt_out + 3) >> 2;
-    int cnt = 0;
-    RowBuf rb;
-    rb.init();
-    uint2* nbr2 = reinterpret_cast<uint2*>(e.nbr);
-    uint2 q = (npk > 0) ? pko[pos] : make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
-    for (int p = 0; p < npk; ++p) {
-      const uint2 qn = (p + 1 < npk) ? pko[(size_t)(p + 1) * ostride + pos] : make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
-      if (H4D_PF_FILTER > 0 && p + H4D_PF_FILTER < npk) prefetch_l2(pko + (size_t)(p + H4D_PF_FILTER) * ostride + pos);
-      const int jj[4] = {(int)(q.x & 0xFFFFu), (int)(q.x >> 16), (int)(q.y & 0xFFFFu), (int)(q.y >> 16)};
-      uint4 pj[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) pj[u] = v.pos[jj[u] == kNoAtom ? i : jj[u]];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const bool ok = jj[u] != kNoAtom && fixed_d2(pi, pj[u]) <= R.T_list;
-        rb.put_if(ok, jj[u]);
-        cnt += ok ? 1 : 0;
-        if (rb.n == 4) {
-          if (cnt <= maxn) nbr2[packet_index(e, R, pos, (cnt - 1) >> 2, ltpa)] = rb.packet();
-          rb.init();
-        }
-      }
-      q = qn;
-    }
-    if (rb.n > 0 && cnt <= maxn) nbr2[packet_index(e, R, pos, (cnt - 1) >> 2, ltpa)] = rb.packet();
-    if (cnt > maxn) { overflow = 1; cnt = maxn & ~3; }
-    e.ncnt[R.atom_off + pos] = cnt;
-    e.ref[R.atom_off + i] = pi;
-  }
+  const int overflow = c.ltpa == 0 ? filter_rows<true>(c, n, lay) : filter_rows<false>(c, n, lay);
   if (overflow) atomicOr(&v.s->flag_overflow, 1);
   c.sync();
   if (c.tid == 0) v.s->n_ord = lay ? n : 0;
@@ -857,7 +878,7 @@ __device__ H4D_PHASE void filter_list_impl(const Ctx& cref) {
 // Coulomb form (pair_fr_lj2_poly) over the erfc form (pair_fr_lj2).
 template <bool NEMD, bool POLY>
 __device__ __forceinline__ void lj_row(const Pot& P, const uint4* __restrict__ pos, const uint2* pk, size_t pstride,
-                                       int npk, uint2 q, unsigned capa, int i, const uint4& pi, float scale, float wi,
+                                       int npk, uint2 q, int i, const uint4& pi, float scale, float wi,
                                        bool wnz_i, float gscr, float& fx, float& fy, float& fz) {
   const unsigned kq_i = __float_as_uint(P.kq[0]) ^ ((unsigned)i << 31);
   for (int p = 0; p < npk; ++p) {
@@ -866,7 +887,7 @@ __device__ __forceinline__ void lj_row(const Pot& P, const uint4* __restrict__ p
     const unsigned jw[4] = {q.x & 0xFFFFu, q.x >> 16, q.y & 0xFFFFu, q.y >> 16};
     uint4 pj[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) pj[u] = pos[min(jw[u], capa)];
+    for (int u = 0; u < 4; ++u) pj[u] = pos[jw[u]];
 #pragma unroll
     for (int h = 0; h < 4; h += 2) {  // slots h and h+1 on the packed FP32x2 pipe
       const float2 dx = __fmul2_rn(make_float2((float)(int)(pj[h].x - pi.x), (float)(int)(pj[h + 1].x - pi.x)), f2(scale));
@@ -960,21 +981,21 @@ __device__ H4D_PHASE void force_pass_impl(const Ctx& cref, int mode, float w_pre
       uint2 q = (npk > 0) ? pk[0] : make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
       if (SYS == H4D_SYS_LJ) {
         if (P.coul_poly)
-          lj_row<NEMD, true>(P, v.pos, pk, pstride, npk, q, (unsigned)R.cap_atoms, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
+          lj_row<NEMD, true>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
         else
-          lj_row<NEMD, false>(P, v.pos, pk, pstride, npk, q, (unsigned)R.cap_atoms, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
+          lj_row<NEMD, false>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
       } else
       for (int p = 0; p < npk; ++p) {
         const uint2 qn = (p + 1 < npk) ? pk[(size_t)(p + 1) * pstride] : make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
         const int jj[4] = {(int)(q.x & 0xFFFFu), (int)(q.x >> 16), (int)(q.y & 0xFFFFu), (int)(q.y >> 16)};
-        // branch-free over the four slots: a padding slot reads atom i and gets r^2 = 1e30,
-        // for which every term of the pair function is exactly zero
+        // branch-free over the four slots: a padding slot (the sentinel) gets r^2 = 1e30, for
+        // which every term of the pair function is exactly zero
         uint4 pj[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) pj[u] = v.pos[jj[u] == kNoAtom ? i : jj[u]];
+        for (int u = 0; u < 4; ++u) pj[u] = v.pos[jj[u]];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const bool valid = jj[u] != kNoAtom;
+          const bool valid = jj[u] != R.cap_atoms;
           const float dx = (float)(int)(pj[u].x - pi.x) * scale;
           const float dy = (float)(int)(pj[u].y - pi.y) * scale;
           const float dz = (float)(int)(pj[u].z - pi.z) * scale;
