@@ -340,8 +340,8 @@ class Context:
 
     def h4d_get_state(self, r=0):
         cap = self.cap_atoms[r]
-        x = np.zeros((cap, 3))
-        v = np.zeros((cap, 3))
+        x = np.empty((cap, 3))
+        v = np.empty((cap, 3))
         n = ctypes.c_int64()
         _ck(lib().h4d_get_state(self.h, r, _pd(x), _pd(v), cap, ctypes.byref(n)), "h4d_get_state")
         return x[: n.value].copy(), v[: n.value].copy()
