@@ -509,8 +509,7 @@ static void set_rep_geometry(const h4d_params& p, Rep& r, double L) {
   r.skin_out_fx = (float)(outer_skin(p) / L * kTwo32);
 }
 
-// every device buffer of a context from one allocation (a cudaMalloc each cost more than half of
-// h4d_create on small systems: 0.37 -> @CREATE@ ms for 250 ions)
+// every device buffer of a context from one allocation
 static int alloc_all(h4d_ctx* c) {
   const size_t na = (size_t)c->total_atoms;
   size_t nrec = 0;
