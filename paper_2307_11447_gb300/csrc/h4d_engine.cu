@@ -71,6 +71,14 @@ __device__ __forceinline__ void ff_scale(float& hi, float& lo, float a) {
   hi = t;
 }
 
+// 1/sqrt without the rescaling of subnormal arguments that rsqrtf adds: squared distances on
+// the 32-bit position grid are far above them
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 __device__ __forceinline__ float wbits(const uint4& p) { return __uint_as_float(p.w); }
 
 // Abramowitz & Stegun 7.1.26: erfc(x) = t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) e^{-x^2},
@@ -138,7 +146,7 @@ __device__ __forceinline__ PairCoef<SYS> coef(const Pot& P, int ti, int tj) {
 // -du/dr / r of the 4D pair term (FP32): LJ (Eq. 19) + screened erfc Coulomb (Eqs. 9-11, 20)
 template <int SYS>
 __device__ __forceinline__ float pair_fr(const Pot& P, const PairCoef<SYS>& c, float r2, float g) {
-  float rinv = rsqrtf(r2);
+  float rinv = rsqrt_approx(r2);
   float rinv2 = rinv * rinv;
   float s2 = c.sig2 * rinv2;
   float s6 = s2 * s2 * s2;
@@ -182,7 +190,7 @@ __device__ __forceinline__ float rcp_approx(float y) {
   return r;
 }
 __device__ __forceinline__ float2 pair_fr_lj2(const Pot& P, float2 r2, float2 kqg) {
-  const float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+  const float2 rinv = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
   const float2 rinv2 = __fmul2_rn(rinv, rinv);
   const float2 s2 = __fmul2_rn(f2(P.sig2[0]), rinv2);
   const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
@@ -208,24 +216,19 @@ __device__ __forceinline__ float2 pair_fr_lj2(const Pot& P, float2 r2, float2 kq
 // The same two pair terms with the screened-Coulomb force as r^-3 + C(r^2) (C the degree-7
 // polynomial the host interpolates for this alpha and cut-off, Pot::cpoly): Eqs. 9-11 with
 // the erfc and Gaussian terms folded into C, so one rsqrt is the only special function of
-// a pair.  The LJ term of Eq. 19 takes 12 eps4 and 6 eps4 as constants.  Pairs beyond a
-// cut-off (skin entries, the sentinel at infinite altitude) are dropped by selects, so the
-// polynomial's value there does not matter.
-__device__ __forceinline__ float2 pair_fr_lj2_poly(const Pot& P, float2 r2, float2 kqg) {
-  const float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+// a pair.  The LJ term of Eq. 19 takes 12 eps4 and 6 eps4 as constants.  Both terms are
+// returned without their cut-offs, which the caller applies; the polynomial's value beyond
+// them (skin entries, the sentinel at infinite altitude) does not matter.
+__device__ __forceinline__ void pair_fr_lj2_poly(const Pot& P, float2 r2, float2 kqg, float2& fr_lj, float2& fr_c) {
+  const float2 rinv = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
   const float2 rinv2 = __fmul2_rn(rinv, rinv);
   const float2 s2 = __fmul2_rn(f2(P.sig2[0]), rinv2);
   const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
-  float2 fr_lj = __fmul2_rn(__fmul2_rn(s6, __ffma2_rn(f2(P.lj12), s6, f2(-P.lj6))), rinv2);
-  fr_lj.x = (r2.x < P.rc2_lj) ? fr_lj.x : 0.0f;
-  fr_lj.y = (r2.y < P.rc2_lj) ? fr_lj.y : 0.0f;
+  fr_lj = __fmul2_rn(__fmul2_rn(s6, __ffma2_rn(f2(P.lj12), s6, f2(-P.lj6))), rinv2);
   float2 cp = __ffma2_rn(f2(P.cpoly[7]), r2, f2(P.cpoly[6]));
 #pragma unroll
   for (int k = 5; k >= 0; --k) cp = __ffma2_rn(cp, r2, f2(P.cpoly[k]));
-  float2 fr_c = __fmul2_rn(kqg, __ffma2_rn(rinv2, rinv, cp));
-  fr_c.x = (r2.x < P.rc2_c) ? fr_c.x : 0.0f;
-  fr_c.y = (r2.y < P.rc2_c) ? fr_c.y : 0.0f;
-  return __fadd2_rn(fr_lj, fr_c);
+  fr_c = __fmul2_rn(kqg, __ffma2_rn(rinv2, rinv, cp));
 }
 
 // FP32 pair energy (protocol-work diagnostic only)
@@ -874,9 +877,16 @@ __device__ H4D_PHASE void filter_list_impl(const Ctx& cref) {
 // slots per packet, pair terms two at a time on the packed FP32x2 pipe.  Padding slots read
 // the sentinel (its infinite altitude puts it beyond every cut-off), and the charge sign of
 // a pair is the parity of i + j (cations even, anions odd): the same values as the generic
-// loop, with neither a branch nor a table load per slot.  POLY selects the polynomial
-// Coulomb form (pair_fr_lj2_poly) over the erfc form (pair_fr_lj2).
-template <bool NEMD, bool POLY>
+// loop, with neither a branch nor a table load per slot.  FORM selects the Coulomb term: the
+// erfc form (0, pair_fr_lj2) or the polynomial (pair_fr_lj2_poly) with the LJ cut-off inside
+// the Coulomb one (1) or beyond it (2).
+// Bound: issue slots and latency together (59% of the slots issue; FMA pipe 57%, shared-memory
+// gathers 57%, ALU 36% busy).  With the LJ cut-off inside, a pair beyond it skips the addition
+// of the LJ term and one beyond both skips the three force sums, all predicated; selecting
+// zeros instead took four instructions more per pair, and rsqrtf's rescaling of subnormal
+// arguments three.  The results are the same bits: adding a zero term changes no sum.  Force
+// passes of 304 chains of 4000 ions inside the engine: 218 -> 207 us.
+template <bool NEMD, int FORM>
 __device__ __forceinline__ void lj_row(const Pot& P, const uint4* __restrict__ pos, const uint2* pk, size_t pstride,
                                        int npk, uint2 q, int i, const uint4& pi, float scale, float wi,
                                        bool wnz_i, float gscr, float& fx, float& fy, float& fz) {
@@ -895,7 +905,8 @@ __device__ __forceinline__ void lj_row(const Pot& P, const uint4* __restrict__ p
       const float2 dz = __fmul2_rn(make_float2((float)(int)(pj[h].z - pi.z), (float)(int)(pj[h + 1].z - pi.z)), f2(scale));
       float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
       const float2 wj = make_float2(wbits(pj[h]), wbits(pj[h + 1]));  // 0, a flyer's altitude, or +inf
-      float2 kqg = make_float2(__uint_as_float(kq_i ^ (jw[h] << 31)), __uint_as_float(kq_i ^ (jw[h + 1] << 31)));
+      // (adding 2^31 flips the sign)
+      float2 kqg = make_float2(__uint_as_float(kq_i + (jw[h] << 31)), __uint_as_float(kq_i + (jw[h + 1] << 31)));
       if (NEMD) {
         const float2 dw = __fadd2_rn(f2(wi), make_float2(-wj.x, -wj.y));
         r2 = __ffma2_rn(dw, dw, r2);
@@ -905,14 +916,32 @@ __device__ __forceinline__ void lj_row(const Pot& P, const uint4* __restrict__ p
       } else {
         r2 = __ffma2_rn(wj, wj, r2);  // + 0 for every atom, +inf for the sentinel
       }
-      const float2 fr = POLY ? pair_fr_lj2_poly(P, r2, kqg) : pair_fr_lj2(P, r2, kqg);
+      float2 fr, fr_c;
+      if (FORM == 0) {
+        fr = pair_fr_lj2(P, r2, kqg);
+      } else {
+        pair_fr_lj2_poly(P, r2, kqg, fr, fr_c);
+        if (FORM == 1) {
+          const float2 lj = fr;
+          fr = fr_c;
+          if (r2.x < P.rc2_lj) fr.x += lj.x;
+          if (r2.y < P.rc2_lj) fr.y += lj.y;
+        } else {
+          fr.x = (r2.x < P.rc2_lj ? fr.x : 0.0f) + (r2.x < P.rc2_c ? fr_c.x : 0.0f);
+          fr.y = (r2.y < P.rc2_lj ? fr.y : 0.0f) + (r2.y < P.rc2_c ? fr_c.y : 0.0f);
+        }
+      }
       // the force sums in slot order, as in the generic loop
-      fx = fmaf(-fr.x, dx.x, fx);
-      fy = fmaf(-fr.x, dy.x, fy);
-      fz = fmaf(-fr.x, dz.x, fz);
-      fx = fmaf(-fr.y, dx.y, fx);
-      fy = fmaf(-fr.y, dy.y, fy);
-      fz = fmaf(-fr.y, dz.y, fz);
+      if (FORM != 1 || r2.x < P.rc2_c) {
+        fx = fmaf(-fr.x, dx.x, fx);
+        fy = fmaf(-fr.x, dy.x, fy);
+        fz = fmaf(-fr.x, dz.x, fz);
+      }
+      if (FORM != 1 || r2.y < P.rc2_c) {
+        fx = fmaf(-fr.y, dx.y, fx);
+        fy = fmaf(-fr.y, dy.y, fy);
+        fz = fmaf(-fr.y, dz.y, fz);
+      }
     }
     q = qn;
   }
@@ -980,10 +1009,12 @@ __device__ H4D_PHASE void force_pass_impl(const Ctx& cref, int mode, float w_pre
       const int npk = (nP > lin) ? (nP - lin + tpa - 1) >> ltpa : 0;
       uint2 q = (npk > 0) ? pk[0] : make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
       if (SYS == H4D_SYS_LJ) {
-        if (P.coul_poly)
-          lj_row<NEMD, true>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
+        if (P.coul_poly && P.rc2_lj <= P.rc2_c)
+          lj_row<NEMD, 1>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
+        else if (P.coul_poly)
+          lj_row<NEMD, 2>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
         else
-          lj_row<NEMD, false>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
+          lj_row<NEMD, 0>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
       } else
       for (int p = 0; p < npk; ++p) {
         const uint2 qn = (p + 1 < npk) ? pk[(size_t)(p + 1) * pstride] : make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
@@ -1448,8 +1479,7 @@ __device__ double energy64(const Ctx& c, int ex0, int ex1, int ex2 = -1) {
 __device__ __forceinline__ double pair_add64(const Pot& P, const CoulPiece* __restrict__ tab, int k, double r2, double kqg,
                                              bool lj, bool co, double part) {
   const float sf = (float)r2;
-  float y0;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(sf));
+  const float y0 = rsqrt_approx(sf);
   // r2 = 0 (two atoms on one grid point): 1/r is infinite, as r2 / r2 arithmetic has it
   const double yd = sf > 1.2e-38f ? f2d_pos(y0) : __hiloint2double(0x7FF00000, 0);
   // e = 1 - r2 y0^2 is below 4e-7: 1/r = y0 (1 + e/2 + 3/8 e^2), the next term below 2e-20
