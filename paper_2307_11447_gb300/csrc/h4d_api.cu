@@ -50,19 +50,19 @@ struct PropDev {
   int* n_valid = nullptr;
   float* bfeat = nullptr;
   float* btgt = nullptr;
-  uint16_t *xT = nullptr, *h1T = nullptr, *dz1T = nullptr, *h2T = nullptr, *dz2T = nullptr, *dlT = nullptr;
-  float* loss_rows = nullptr;
+  float* part = nullptr;        // partial gradients and losses, one per CTA
+  double* part_loss = nullptr;
   double* loss = nullptr;
   float* fout = nullptr;  // [cells][96] feature dump of h4d_proposal_logits
 };
 
 static void prop_free_train(PropDev* P) {
-  void* ptrs[] = {P->bfeat, P->btgt, P->xT, P->h1T, P->dz1T, P->h2T, P->dz2T, P->dlT, P->loss_rows};
+  void* ptrs[] = {P->bfeat, P->btgt, P->part, P->part_loss};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   P->bfeat = P->btgt = nullptr;
-  P->xT = P->h1T = P->dz1T = P->h2T = P->dz2T = P->dlT = nullptr;
-  P->loss_rows = nullptr;
+  P->part = nullptr;
+  P->part_loss = nullptr;
   P->cap_rows = 0;
 }
 
@@ -99,21 +99,17 @@ static int prop_alloc_net(PropDev* P) {
   return H4D_OK;
 }
 
-// training scratch for `rows` rows (a multiple of 16)
+// training scratch for `rows` rows
 static int prop_ensure_rows(PropDev* P, int rows) {
   if (rows <= P->cap_rows) return H4D_OK;
   prop_free_train(P);
-  const size_t r = (size_t)rows;
+  const size_t r = (size_t)rows, parts = (size_t)prop_grad_parts(rows);
   CKP(cudaMalloc(&P->bfeat, r * 96 * sizeof(float)));
   CKP(cudaMalloc(&P->btgt, r * sizeof(float)));
-  CKP(cudaMalloc(&P->xT, 96 * r * sizeof(uint16_t)));
-  CKP(cudaMalloc(&P->h1T, 64 * r * sizeof(uint16_t)));
-  CKP(cudaMalloc(&P->dz1T, 64 * r * sizeof(uint16_t)));
-  CKP(cudaMalloc(&P->h2T, 64 * r * sizeof(uint16_t)));
-  CKP(cudaMalloc(&P->dz2T, 64 * r * sizeof(uint16_t)));
-  CKP(cudaMalloc(&P->dlT, 8 * r * sizeof(uint16_t)));
-  CKP(cudaMalloc(&P->loss_rows, r * sizeof(float)));
-  CKP(cudaMemset(P->dlT, 0, 8 * r * sizeof(uint16_t)));  // rows 2..7 of dl stay zero
+  // fewer rows can need more CTAs than these (whole blocks per CTA), never more than 152
+  const size_t cap = rows <= 152 * 128 ? parts : 152;
+  CKP(cudaMalloc(&P->part, cap * kPropNW * sizeof(float)));
+  CKP(cudaMalloc(&P->part_loss, cap * sizeof(double)));
   P->cap_rows = rows;
   return H4D_OK;
 }
@@ -124,13 +120,9 @@ static PropNet prop_net(const PropDev* P) {
   return n;
 }
 
-// loss and gradient of n records already in P->bfeat / P->btgt (rows_pad rows)
-static int prop_loss_grad(PropDev* P, int n, int rows_pad, cudaStream_t s) {
-  int rc = launch_prop_fwd_bwd(prop_net(P), P->bfeat, P->btgt, n, 1.0f / (float)n, P->xT, P->h1T, P->dz1T, P->h2T,
-                               P->dz2T, P->dlT, P->loss_rows, rows_pad, s);
-  if (rc) return rc;
-  return launch_prop_wgrad(P->xT, P->h1T, P->dz1T, P->h2T, P->dz2T, P->dlT, P->loss_rows, rows_pad, P->grad,
-                           P->loss, s);
+// loss and gradient of n records already in P->bfeat / P->btgt
+static int prop_loss_grad(PropDev* P, int n, cudaStream_t s) {
+  return launch_prop_grad(prop_net(P), P->bfeat, P->btgt, n, 1.0f / (float)n, P->part, P->part_loss, P->grad, P->loss, s);
 }
 
 struct h4d_ctx {
@@ -1991,14 +1983,13 @@ int h4d_train_proposal(h4d_ctx* c, int64_t steps, int32_t batch, double lr, doub
   CK(cudaStreamSynchronize(c->stream));
   if (n_valid == 0) return H4D_EINVAL;
   const int nb = std::min(batch, n_valid);
-  const int rows_pad = ((2 * nb + 15) / 16) * 16;
-  rc = prop_ensure_rows(P, rows_pad);
+  rc = prop_ensure_rows(P, 2 * nb);
   if (rc) return rc;
   for (int64_t s = 0; s < steps; ++s) {
     rc = launch_prop_gather(P->rfeat, P->ry, P->valid, n_valid, nb, seed, (long long)P->adam_t, (float)y0, P->bfeat,
                             P->btgt, c->stream);
     if (rc) return rc;
-    rc = prop_loss_grad(P, nb, rows_pad, c->stream);
+    rc = prop_loss_grad(P, nb, c->stream);
     if (rc) return rc;
     P->adam_t++;
     rc = launch_prop_adam(P->w, P->m, P->v, P->grad, (int)std::min<long long>(P->adam_t, 1 << 30), (float)lr,
@@ -2028,18 +2019,17 @@ int h4d_proposal_grad(const double* w, int64_t n_rec, const float* feat, const f
   if (!P) return H4D_ECUDA;
   cudaStream_t s = 0;
   const int n = (int)n_rec;
-  const int rows_pad = ((2 * n + 15) / 16) * 16;
   std::vector<float> f(kPropNW);
   for (int i = 0; i < kPropNW; ++i) f[i] = (float)w[i];
   rc = prop_alloc_net(P);
-  if (!rc) rc = prop_ensure_rows(P, rows_pad);
+  if (!rc) rc = prop_ensure_rows(P, 2 * n);
   if (!rc && cudaMemcpy(P->w, f.data(), kPropNW * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) rc = H4D_ECUDA;
   if (!rc && cudaMemcpy(P->bfeat, feat, (size_t)n * 192 * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
     rc = H4D_ECUDA;
   if (!rc && cudaMemcpy(P->btgt, tgt, (size_t)n * 2 * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
     rc = H4D_ECUDA;
   if (!rc) rc = prop_pack(P, s);
-  if (!rc) rc = prop_loss_grad(P, n, rows_pad, s);
+  if (!rc) rc = prop_loss_grad(P, n, s);
   double l = 0.0;
   if (!rc && cudaMemcpy(&l, P->loss, sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess) rc = H4D_ECUDA;
   if (!rc && cudaMemcpy(f.data(), P->grad, kPropNW * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)

@@ -127,13 +127,12 @@ __device__ __forceinline__ void mlp_tile_forward(const PropNet& net, LoadA loadA
 // Launches of the proposal kernels (h4d_train.cu)
 int launch_prop_pack(const float* w, uint2* w1, uint2* w2, uint2* w3, uint2* w2t, float* w3r, float* b,
                      void* stream);
-// rows = 2 * n_rec (cation row then anion row of each record); targets t[n_rec][2]
-int launch_prop_fwd_bwd(const PropNet& net, const float* feat, const float* tgt, int n_rec, float inv_n,
-                        uint16_t* xT, uint16_t* h1T, uint16_t* dz1T, uint16_t* h2T, uint16_t* dz2T,
-                        uint16_t* dlT, float* loss_rows, int rows_pad, void* stream);
-int launch_prop_wgrad(const uint16_t* xT, const uint16_t* h1T, const uint16_t* dz1T, const uint16_t* h2T,
-                      const uint16_t* dz2T, const uint16_t* dlT, const float* loss_rows, int rows_pad,
-                      float* grad, double* loss, void* stream);
+// loss (summed over records) and its gradient; rows = 2 * n_rec (cation row then anion row of
+// each record), targets t[n_rec][2]; part [parts][kPropNW] and part_loss [parts] with
+// parts = prop_grad_parts(rows)
+int prop_grad_parts(int rows);
+int launch_prop_grad(const PropNet& net, const float* feat, const float* tgt, int n_rec, float inv_n, float* part,
+                     double* part_loss, float* grad, double* loss, void* stream);
 int launch_prop_adam(float* w, float* m, float* v, const float* grad, int step, float lr, void* stream);
 // minibatch of n_batch records (uniform draws keyed by (seed, step)), or all valid records
 // in order when n_batch >= n_valid
