@@ -1459,16 +1459,13 @@ int h4d_load(h4d_ctx* c, const char* path) {
 }
 
 // ---- stateless entry points ----
-int h4d_eval_forces(const h4d_params* params, double L, int32_t n_water, int32_t n, const double* x,
-                    const double* w, double* F, double* U) {
-  int rc = check_params(params);
-  if (rc) return rc;
-  if (((!x || !F) && n > 0) || n < 0 || n_water < 0 || 3 * n_water > n || !(L > 0)) return H4D_EINVAL;
-  if (unit_of(*params) == 2 && ((n - 3 * n_water) & 1) != 0) return H4D_EINVAL;
-  if (2.0 * (rmax_of(*params) + params->skin) >= L) return H4D_EINVAL;
-  if (n > 65535) return H4D_ECAPACITY;
-  rc = check_device();
-  if (rc) return rc;
+}  // extern "C"
+
+// h4d_eval_forces through the engine's lists on one CTA: the verdict on systems whose rows come
+// near their capacities
+static int eval_forces_lists(const h4d_params* params, double L, int32_t n_water, int32_t n, const double* x,
+                             const double* w, double* F, double* U) {
+  int rc;
   h4d_ctx* c = new (std::nothrow) h4d_ctx();
   if (!c) return H4D_ECUDA;
   c->prm = *params;
@@ -1527,6 +1524,8 @@ int h4d_eval_forces(const h4d_params* params, double L, int32_t n_water, int32_t
   h4d_destroy(c);
   return rc;
 }
+
+extern "C" {
 
 int h4d_neighbor_pairs(double L, int32_t n, const double* x, double r_list, int32_t* oi, int32_t* oj, int64_t cap,
                        int64_t* n_out) {
@@ -1660,6 +1659,93 @@ static size_t carve_bytes(size_t& off, size_t bytes) {
   const size_t at = (off + 255) & ~(size_t)255;
   off = at + bytes;
   return at;
+}
+
+extern "C" int h4d_eval_forces(const h4d_params* params, double L, int32_t n_water, int32_t n, const double* x,
+                               const double* w, double* F, double* U) {
+  int rc = check_params(params);
+  if (rc) return rc;
+  if (((!x || !F) && n > 0) || n < 0 || n_water < 0 || 3 * n_water > n || !(L > 0)) return H4D_EINVAL;
+  if (unit_of(*params) == 2 && ((n - 3 * n_water) & 1) != 0) return H4D_EINVAL;
+  if (2.0 * (rmax_of(*params) + params->skin) >= L) return H4D_EINVAL;
+  if (n > 65535) return H4D_ECAPACITY;
+  rc = check_device();
+  if (rc) return rc;
+  if (n == 0) {
+    if (U) *U = 0.0;
+    return H4D_OK;
+  }
+  Rep R;
+  std::memset(&R, 0, sizeof(Rep));
+  set_rep_geometry(*params, R, L);
+  if (group_smem_bytes(n, R.nc, 0) > 227 * 1024) return H4D_ECAPACITY;  // as a replica of the engine
+  Point P;
+  Proto pr;
+  std::memset(&P, 0, sizeof(P));
+  fill_pot(*params, P.pot, pr);
+  P.L = L;
+  P.n = n;
+  P.nw3 = 3 * n_water;
+  P.T_list = R.T_list;
+  // what passes the outer lists' conservative tests is within their radius plus one quantum per
+  // axis of the coordinates they run on (8-bit with cells, 16-bit without)
+  const double q = R.nc > 0 ? L / 256.0 : L / 65536.0;
+  const double rq = (std::sqrt((double)(R.nc > 0 ? R.T8_out : R.T16_out)) + 1.7320508075688774) * q / L * kTwo32;
+  P.T_out_max = (unsigned long long)(rq * rq);
+  P.max_nbr = params->max_nbr > 0 ? params->max_nbr : derive_max_nbr(*params);
+  P.max_nbr = ((P.max_nbr + 127) / 128) * 128;
+  P.max_out = std::max(P.max_nbr, derive_max_rows(*params, rmax_of(*params) + outer_skin(*params)));
+  double wsum = 0.0;
+  int wcnt = 0;
+  if (w)
+    for (int a = 0; a < n; ++a)
+      if ((float)w[a] != 0.0f) { wsum += w[a]; ++wcnt; }
+  P.wbar = (float)(wcnt ? wsum / wcnt : 0.0);
+  int warps, ctas;
+  const int n_part = point_plan(n, &warps, &P.homes, &ctas);
+  const std::vector<CoulPiece> tab = coul_table(params->alpha, params->rc_coul);
+  // one allocation; inputs and results are each one piece
+  const size_t na = (size_t)n;
+  size_t off = 0;
+  const size_t o_x = carve_bytes(off, na * 3 * sizeof(double));
+  const size_t o_w = carve_bytes(off, w ? na * sizeof(double) : 0);
+  const size_t o_tab = carve_bytes(off, tab.size() * sizeof(CoulPiece));
+  const size_t o_pos = carve_bytes(off, na * sizeof(uint4));
+  const size_t n_out = 1 + (size_t)n_part + 3 * na;
+  const size_t o_out = carve_bytes(off, n_out * sizeof(double));
+  unsigned char* b = nullptr;
+  CK(cudaMalloc(&b, off));
+  double* out = reinterpret_cast<double*>(b + o_out);  // overflow flag, energy partials, forces
+  P.pos = reinterpret_cast<const uint4*>(b + o_pos);
+  P.etab = reinterpret_cast<const CoulPiece*>(b + o_tab);
+  P.may_overflow = out;
+  P.u_part = out + 1;
+  P.F = out + 1 + n_part;
+  std::vector<double> res(n_out);
+  auto ok = [](cudaError_t e) { return e == cudaSuccess; };
+  bool good = ok(cudaMemcpyAsync(b + o_x, x, na * 3 * sizeof(double), cudaMemcpyHostToDevice, 0));
+  if (w) good = good && ok(cudaMemcpyAsync(b + o_w, w, na * sizeof(double), cudaMemcpyHostToDevice, 0));
+  good = good && ok(cudaMemcpyAsync(b + o_tab, tab.data(), tab.size() * sizeof(CoulPiece), cudaMemcpyHostToDevice, 0));
+  good = good && ok(cudaMemsetAsync(out, 0, sizeof(double), 0));
+  if (good) {
+    static_convert_in<<<(n + 255) / 256, 256>>>(reinterpret_cast<const double*>(b + o_x),
+                                                 w ? reinterpret_cast<const double*>(b + o_w) : nullptr, n, L,
+                                                 reinterpret_cast<uint4*>(b + o_pos));
+    good = ok(cudaGetLastError()) && launch_point(P, warps, ctas, 0) == H4D_OK;
+  }
+  good = good && ok(cudaMemcpy(res.data(), out, n_out * sizeof(double), cudaMemcpyDeviceToHost));
+  cudaFree(b);
+  if (!good) return H4D_ECUDA;
+  if (res[0] != 0.0) return eval_forces_lists(params, L, n_water, n, x, w, F, U);
+  double u = 0.0, comp = 0.0;
+  for (int k = 0; k < n_part; ++k) {
+    const double y = res[1 + k] - comp, t = u + y;
+    comp = (t - u) - y;
+    u = t;
+  }
+  if (U) *U = u;
+  std::memcpy(F, res.data() + 1 + n_part, 3 * na * sizeof(double));
+  return H4D_OK;
 }
 
 extern "C" int h4d_eval_forces_static(const h4d_params* params, double L, int32_t n_water, int32_t n,

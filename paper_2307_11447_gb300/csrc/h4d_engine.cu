@@ -2908,6 +2908,176 @@ int launch_eval(const Eng& e, int threads, size_t smem, float wbar, double* U, v
   return cudaGetLastError() == cudaSuccess ? H4D_OK : H4D_ECUDA;
 }
 
+// ------------------------------------------------------------------------------------
+// Single-point forces and energy of one configuration over the whole GPU
+// ------------------------------------------------------------------------------------
+// A warp per home atom (kHomes of them in turn): it runs over all atoms, 32 per step, with the
+// exact integer distance test, and queues the ones inside the cut-off in shared memory, pairs
+// whose energy this atom owns apart from the others; a full queue of 32 is one FP32 force term
+// per lane and, for the owned pairs, one FP64 energy term, so no lane of the slow FP64 pipe
+// idles.  All positions sit in shared memory.  No list is built: testing all pairs costs less
+// than sorting at these sizes (n^2 / 32 tests of about 30 cycles over 608 schedulers, 0.1 ms at
+// 9110 atoms).  The lists' capacities are still part of the call: two counts per home bound the
+// rows that the list build would make, and the host takes that path when a row could overflow.
+// Calls of h4d_eval_forces: 2.9 ms for 1000 ions and 13.9 ms for 400 waters with the engine's lists
+// on one CTA, 0.30 and 0.26 ms with this kernel.
+struct TwoF {  // unevaluated sum
+  float hi, lo;
+};
+__device__ __forceinline__ TwoF two_add(TwoF a, TwoF b) {
+  const float s = a.hi + b.hi, bp = s - a.hi;
+  const float e = (a.hi - (s - bp)) + (b.hi - bp);
+  return TwoF{s, e + (a.lo + b.lo)};
+}
+__device__ __forceinline__ float warp_sum2(float hi, float lo) {
+  TwoF v{hi, lo};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    v = two_add(v, TwoF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+  return v.hi + v.lo;
+}
+
+template <int SYS>
+__global__ void __launch_bounds__(512) point_kernel(const __grid_constant__ Point a) {
+  extern __shared__ __align__(16) char smem[];
+  uint4* pos = reinterpret_cast<uint4*>(smem);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  // two queues of up to 63 + 32 entries per warp (owned pairs, other pairs)
+  uint16_t* queue = reinterpret_cast<uint16_t*>(smem + 16 * (size_t)a.n) + 192 * warp;
+  for (int k = threadIdx.x; k < a.n; k += blockDim.x) pos[k] = a.pos[k];
+  __syncthreads();
+  const Pot& P = a.pot;
+  const float scale = (float)(a.L / 4294967296.0);
+  const double dscale = a.L * 0x1.0p-32, scale2 = dscale * dscale;
+  const float gscr = expf(-P.kappa_sr * a.wbar);
+  const double gscr64 = exp(-P.dkappa_sr * (double)a.wbar);
+  const u64 T_lj = (u64)ceil(P.drc2_lj / scale2), T_c = (u64)ceil(P.drc2_c / scale2);
+  const u64 T_max = T_lj > T_c ? T_lj : T_c;
+  const unsigned lt = (1u << lane) - 1u;
+  const int w0 = (blockIdx.x * nwarps + warp) * a.homes;
+  double part = 0.0;
+  for (int i = w0; i < min(w0 + a.homes, a.n); ++i) {
+    const uint4 pi = pos[i];
+    const int ti = type_t<SYS>(i, a.nw3);
+    const float wi = wbits(pi);
+    const unsigned ex0 = i < a.nw3 ? (unsigned)(i - i % 3) : (unsigned)i, exn = i < a.nw3 ? 3u : 1u;
+    float fx = 0.f, fy = 0.f, fz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;  // compensated sums
+    int n_out = 0, n_list = 0;
+    int nq[2] = {0, 0};
+    // the first m (at most 32) entries of queue q
+    auto evaluate = [&](int q, int m) {
+      __syncwarp();
+      if (lane < m) {
+        const int j = queue[96 * q + lane];
+        const uint4 pj = pos[j];
+        const float wj = wbits(pj);
+        const float dx = (float)(int)(pj.x - pi.x) * scale, dy = (float)(int)(pj.y - pi.y) * scale,
+                    dz = (float)(int)(pj.z - pi.z) * scale, dw = wi - wj;
+        const float r2 = fmaf(dw, dw, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+        const bool screened = (wi != 0.f) != (wj != 0.f);
+        const int tj = type_t<SYS>(j, a.nw3);
+        const PairCoef<SYS> cf = coef<SYS>(P, ti, tj);
+        float fr;
+        if (SYS == H4D_SYS_LJ && P.coul_poly) {
+          const float kqg = cf.kq * (screened ? gscr : 1.0f);
+          float2 lj, co;
+          pair_fr_lj2_poly(P, f2(r2), f2(kqg), lj, co);
+          fr = (r2 < P.rc2_lj ? lj.x : 0.0f) + (r2 < P.rc2_c ? co.x : 0.0f);
+        } else {
+          fr = pair_fr<SYS>(P, cf, r2, screened ? gscr : 1.0f);
+        }
+        const float tx = -fr * dx - cx, ty = -fr * dy - cy, tz = -fr * dz - cz;
+        const float sx = fx + tx, sy = fy + ty, sz = fz + tz;
+        cx = (sx - fx) - tx;
+        cy = (sy - fy) - ty;
+        cz = (sz - fz) - tz;
+        fx = sx;
+        fy = sy;
+        fz = sz;
+        if (q == 0) {
+          const int tk = ti * 4 + tj;
+          const u64 d2 = fixed_d2(pi, pj);
+          double r264 = __ull2double_rn(d2) * scale2;
+          double kqg = P.dkq[tk];
+          bool lj = d2 < T_lj, co = d2 < T_c;
+          if (wi != wj) {
+            const double dw64 = (double)wi - (double)wj;
+            r264 = fma(dw64, dw64, r264);
+            lj = r264 < P.drc2_lj;
+            co = r264 < P.drc2_c;
+            if (screened) kqg *= gscr64;
+          }
+          if (P.etab_n > 0) part = pair_add64(P, a.etab, tk, r264, kqg, lj, co, part);
+          else part += pair_u64(P, ti, tj, r264, screened ? gscr64 : 1.0);
+        }
+      }
+      __syncwarp();
+    };
+    auto push = [&](int q, bool ok, int j) {
+      const unsigned m = __ballot_sync(0xffffffffu, ok);
+      if (m == 0u) return;
+      if (ok) queue[96 * q + nq[q] + __popc(m & lt)] = (uint16_t)j;
+      nq[q] += __popc(m);
+      if (nq[q] >= 32) {
+        evaluate(q, 32);
+        nq[q] -= 32;  // at most 31 entries move down
+        const uint16_t t = lane < nq[q] ? queue[96 * q + 32 + lane] : (uint16_t)0;
+        __syncwarp();
+        if (lane < nq[q]) queue[96 * q + lane] = t;
+        __syncwarp();
+      }
+    };
+    for (int q0 = 0; q0 < a.n; q0 += 32) {
+      const int j = min(q0 + lane, a.n - 1);
+      const u64 d2 = fixed_d2(pi, pos[j]);
+      const bool valid = q0 + lane < a.n;
+      n_out += valid && d2 <= a.T_out_max ? 1 : 0;
+      n_list += valid && d2 <= a.T_list ? 1 : 0;
+      const bool in = valid && d2 < T_max && (unsigned)j - ex0 >= exn;
+      if (!__any_sync(0xffffffffu, in)) continue;
+      const bool own = ((i ^ j) & 1) ? i < j : i > j;
+      push(0, in && own, j);
+      push(1, in && !own, j);
+    }
+    evaluate(0, nq[0]);
+    evaluate(1, nq[1]);
+    const float sx = warp_sum2(fx, -cx), sy = warp_sum2(fy, -cy), sz = warp_sum2(fz, -cz);
+    n_out = __reduce_add_sync(0xffffffffu, n_out);
+    n_list = __reduce_add_sync(0xffffffffu, n_list);
+    if (lane == 0) {
+      a.F[3 * i] = sx;
+      a.F[3 * i + 1] = sy;
+      a.F[3 * i + 2] = sz;
+      if (n_out > a.max_out || n_list > a.max_nbr) *a.may_overflow = 1.0;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  if (lane == 0) a.u_part[blockIdx.x * nwarps + warp] = part;
+}
+
+// warps per CTA and homes per warp: about one wave of 16 warps per SM, with 8-warp CTAs while
+// those alone do not cover the SMs twice (1000 ions: 125 CTAs instead of 63)
+int point_plan(int n, int* warps, int* homes, int* ctas) {
+  *homes = (n + 152 * 16 - 1) / (152 * 16);
+  *warps = n <= 152 * 16 ? 8 : 16;
+  *ctas = (n + *warps * *homes - 1) / (*warps * *homes);
+  return *warps * *ctas;
+}
+
+int launch_point(const Point& a, int warps, int ctas, void* stream) {
+  cudaStream_t st = (cudaStream_t)stream;
+  const size_t smem = 16 * (size_t)a.n + 384 * (size_t)warps;
+  if (a.pot.sys == H4D_SYS_LJ) {
+    cudaFuncSetAttribute(point_kernel<H4D_SYS_LJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    point_kernel<H4D_SYS_LJ><<<ctas, 32 * warps, smem, st>>>(a);
+  } else {
+    cudaFuncSetAttribute(point_kernel<H4D_SYS_AQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    point_kernel<H4D_SYS_AQ><<<ctas, 32 * warps, smem, st>>>(a);
+  }
+  return cudaGetLastError() == cudaSuccess ? H4D_OK : H4D_ECUDA;
+}
+
 // n_iter equilibrium force passes on the current state (autotuning and profiling of the
 // pair term in isolation); leaves positions and velocities untouched
 template <int SYS>

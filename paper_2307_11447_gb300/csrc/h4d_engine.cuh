@@ -163,6 +163,23 @@ struct Eng {
   const CoulPiece* etab;  // FP64 Coulomb table (pot.etab_n pieces)
 };
 
+// One configuration for the single-point kernel
+struct Point {
+  Pot pot;
+  double L;
+  int n, nw3, homes;     // atoms, atoms of waters, home atoms per warp
+  float wbar;            // mean altitude of the flying particles
+  unsigned long long T_list, T_out_max;  // Verlet criterion; bound on what the outer test accepts
+  int max_nbr, max_out;  // row capacities of the lists
+  const uint4* pos;
+  const CoulPiece* etab;
+  double* F;             // [n][3]
+  double* u_part;        // energy of each warp's owned pairs
+  double* may_overflow;  // nonzero: a list row could exceed its capacity
+};
+int point_plan(int n, int* warps, int* homes, int* ctas);  // returns the number of warps
+int launch_point(const Point& a, int warps, int ctas, void* stream);
+
 // shared-memory bytes a group needs for a replica
 __host__ __device__ inline size_t smem_align16(size_t b) { return (b + 15) & ~(size_t)15; }
 // Per-group shared memory: positions (plus one sentinel slot after the last atom, which
