@@ -457,6 +457,16 @@ __device__ double fixed_order_sum(const Ctx& c, double* buf, int n) {
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
+// Load of a row packet, left where it is written: ahead of the work on the packet before it
+// (the compiler moved a plain load behind that work, to the next iteration's first use).  Rows
+// stream through once per pass, so they are kept out of L1, where they would push out the
+// velocities that the half kick prefetches.
+__device__ __forceinline__ uint2 ld_packet(const uint2* p) {
+  uint2 q;
+  asm volatile("ld.global.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(q.x), "=r"(q.y) : "l"(p));
+  return q;
+}
+
 __device__ __forceinline__ u64 gtimer() {
   u64 t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
@@ -525,27 +535,29 @@ __device__ void refresh_list(const Ctx& c) {
 }
 // Entries of a lane's row collected in a register pair, first entry lowest: an accepted
 // 16-bit index is shifted in by byte permutes and a full pair is one packet store, all
-// predicated.  The row's packets are cap_atoms apart (outer rows and Verlet rows of one lane)
+// predicated (the store is written as such: left to a branch, an entry cost twice the
+// instructions).  The row's packets are cap_atoms apart (outer rows and Verlet rows of one lane)
 // or, with tpa lanes per Verlet row (T1 false), dealt as packet_index does.
 template <bool T1>
 struct RowOut {
-  uint2* base;    // first packet of the replica
-  unsigned wo;    // offset of the next packet
+  uint2* p;       // next packet
   unsigned cap, tpa;
   int cnt, max;   // entries so far, capacity (a multiple of 4)
   unsigned lo, hi;
-  __device__ __forceinline__ RowOut(uint2* b, unsigned pos, unsigned cap_, unsigned tpa_, int ltpa, int max_)
-      : base(b), wo(pos << (T1 ? 0 : ltpa)), cap(cap_), tpa(tpa_), cnt(0), max(max_), lo(0u), hi(0u) {}
+  __device__ __forceinline__ RowOut(uint2* base, unsigned pos, unsigned cap_, unsigned tpa_, int ltpa, int max_)
+      : p(base + (pos << (T1 ? 0 : ltpa))), cap(cap_), tpa(tpa_), cnt(0), max(max_), lo(0u), hi(0u) {}
   // the entry is the low (sel 0x5432) or the high (0x7632) half of word
   __device__ __forceinline__ void put(bool ok, unsigned word, unsigned sel) {
     lo = ok ? __byte_perm(lo, hi, 0x5432) : lo;
     hi = ok ? __byte_perm(hi, word, sel) : hi;
     cnt += ok ? 1 : 0;
-    if (ok && (cnt & 3) == 0 && cnt <= max) {
-      base[wo] = make_uint2(lo, hi);
-      if (T1) wo += cap;
-      else wo += (((unsigned)cnt >> 2) & (tpa - 1)) ? 1u : cap * tpa - (tpa - 1);
-    }
+    const int full = ok && (cnt & 3) == 0 && cnt <= max;
+    const unsigned step = T1 ? cap : ((((unsigned)cnt >> 2) & (tpa - 1)) ? 1u : cap * tpa - (tpa - 1));
+    asm volatile(
+        "{\n .reg .pred f;\n setp.ne.s32 f, %1, 0;\n @f st.global.v2.u32 [%0], {%2, %3};\n @f add.s64 %0, %0, %4;\n}"
+        : "+l"(p)
+        : "r"(full), "r"(lo), "r"(hi), "l"((unsigned long long)step * sizeof(uint2))
+        : "memory");
   }
   // the last partial packet, completed with pad2 (two entries); true when the row overflowed
   // (cnt is then cut to whole packets)
@@ -555,7 +567,7 @@ struct RowOut {
       uint2 t;
       t.x = r == 1 ? __byte_perm(hi, pad2, 0x5432) : (r == 2 ? hi : __byte_perm(lo, hi, 0x5432));
       t.y = r == 3 ? __byte_perm(hi, pad2, 0x5432) : pad2;
-      base[wo] = t;
+      *p = t;
     }
     if (cnt <= max) return false;
     cnt = max & ~3;
@@ -831,7 +843,8 @@ __device__ __forceinline__ int filter_rows(const Ctx& c, int n, bool lay) {
     const uint2* src = pko + k;
     uint2 q = (npk > 0) ? src[0] : make_uint2(0u, 0u);
     for (int p = 0; p < npk; ++p) {
-      const uint2 qn = (p + 1 < npk) ? src[(size_t)(p + 1) * cap] : make_uint2(0u, 0u);
+      uint2 qn = make_uint2(0u, 0u);
+      if (p + 1 < npk) qn = ld_packet(src + (size_t)(p + 1) * cap);
       if (H4D_PF_FILTER > 0 && p + H4D_PF_FILTER < npk) prefetch_l2(src + (size_t)(p + H4D_PF_FILTER) * cap);
       const int left = cnt_out - 4 * p;  // entries of this packet; the others are not read
       const int j0 = (int)(q.x & 0xFFFFu);
@@ -892,7 +905,8 @@ __device__ __forceinline__ void lj_row(const Pot& P, const uint4* __restrict__ p
                                        bool wnz_i, float gscr, float& fx, float& fy, float& fz) {
   const unsigned kq_i = __float_as_uint(P.kq[0]) ^ ((unsigned)i << 31);
   for (int p = 0; p < npk; ++p) {
-    const uint2 qn = (p + 1 < npk) ? pk[(size_t)(p + 1) * pstride] : make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
+    uint2 qn = make_uint2(0u, 0u);
+    if (p + 1 < npk) qn = ld_packet(pk + (size_t)(p + 1) * pstride);
     if (H4D_PF_FORCE > 0 && p + H4D_PF_FORCE < npk) prefetch_l2(pk + (size_t)(p + H4D_PF_FORCE) * pstride);
     const unsigned jw[4] = {q.x & 0xFFFFu, q.x >> 16, q.y & 0xFFFFu, q.y >> 16};
     uint4 pj[4];
@@ -1017,7 +1031,8 @@ __device__ H4D_PHASE void force_pass_impl(const Ctx& cref, int mode, float w_pre
           lj_row<NEMD, 0>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
       } else
       for (int p = 0; p < npk; ++p) {
-        const uint2 qn = (p + 1 < npk) ? pk[(size_t)(p + 1) * pstride] : make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
+        uint2 qn = make_uint2(0u, 0u);
+        if (p + 1 < npk) qn = ld_packet(pk + (size_t)(p + 1) * pstride);
         const int jj[4] = {(int)(q.x & 0xFFFFu), (int)(q.x >> 16), (int)(q.y & 0xFFFFu), (int)(q.y >> 16)};
         // branch-free over the four slots: a padding slot (the sentinel) gets r^2 = 1e30, for
         // which every term of the pair function is exactly zero
