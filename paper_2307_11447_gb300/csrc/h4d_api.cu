@@ -395,6 +395,8 @@ static void fill_pot(const h4d_params& p, Pot& P, Proto& pr) {
   }
   P.d_oh2 = p.d_oh * p.d_oh;
   P.d_hh2 = p.d_hh * p.d_hh;
+  P.d_oh2_f = (float)P.d_oh2;
+  P.d_hh2_f = (float)P.d_hh2;
   for (int t = 0; t < 4; ++t) P.q[t] = (t < p.ntypes) ? (float)p.q[t] : 0.f;
   P.erfcx_fit = p.alpha * p.rc_coul <= 3.2 ? 1 : 0;  // the fit's range (fit_erfcx.py)
   P.coul_poly = (p.system == H4D_SYS_LJ) ? fit_coul_poly(p.alpha, p.rc_coul, P.cpoly) : 0;
@@ -413,6 +415,7 @@ static void fill_pot(const h4d_params& p, Pot& P, Proto& pr) {
   pr.w_max = p.w_max;
   pr.sched_n = p.sched_n;
   pr.dt = p.dt;
+  pr.dt_f = (float)p.dt;
   pr.tau_t = p.tau_t;
   pr.beta = p.beta;
   pr.beta_mu = p.beta_mu;

@@ -277,7 +277,7 @@ struct GScal {
   int fly2, flyw;              // water exchange: third flying atom, flying water (-1 = none)
   int nw_trial;                // waters in the layout of the running trial
   int n_ord;                   // atoms of the current Verlet-row layout (sorted[0, n_ord)); 0 = by index
-  float w_cur, g_scr, pad2, pad3;
+  float w_cur, g_scr, w_prev, pad3;  // altitude now and before the step
   double alpha_th, dW[3], wprot, wprot_c, red_out;
   double ln_u, ustart, kstart, uend, kend;
   double vfly[6];
@@ -992,7 +992,7 @@ __device__ H4D_PHASE void force_pass_impl(const Ctx& cref, int mode, float w_pre
   const int fly0 = NEMD ? v.s->fly0 : -1, fly1 = NEMD ? v.s->fly1 : -1, fly2 = NEMD ? v.s->fly2 : -1;
   const float gscr = NEMD ? v.s->g_scr : 1.0f;
   const float scale = R.scale;
-  const float half_dt = 0.5f * (float)e.proto.dt;
+  const float half_dt = 0.5f * e.proto.dt_f;
   const uint2* packets = nbr_packets(e, R);
   const size_t pstride = (size_t)R.cap_atoms << ltpa;
   long long kin = 0;  // m v^2 of this thread's atoms, fixed point (exact, order-free sum)
@@ -1152,7 +1152,7 @@ __device__ void water_kick_drift(const Ctx& c, int m, float alpha, float& d1, fl
   const RepC& R = c.r;
   const Pot& P = e.pot;
   const GView& v = c.v;
-  const float h = (float)e.proto.dt;
+  const float h = e.proto.dt_f;
   const float imv[3] = {P.inv_m[2], P.inv_m[3], P.inv_m[3]};  // 1/(m mvv2e): O, H, H
   const float mw[3] = {1.0f / P.inv_m[2], 1.0f / P.inv_m[3], 1.0f / P.inv_m[3]};
   float4 vh[3], vl[3];
@@ -1185,7 +1185,7 @@ __device__ void water_kick_drift(const Ctx& c, int m, float alpha, float& d1, fl
     x[k][2] = ro[k][2] + (vh[k].z + vl[k].z) * h;
   }
   const int ca[3] = {0, 0, 1}, cb[3] = {1, 2, 2};
-  const float dd[3] = {(float)P.d_oh2, (float)P.d_oh2, (float)P.d_hh2};
+  const float dd[3] = {P.d_oh2_f, P.d_oh2_f, P.d_hh2_f};
   float dv[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
   // iterate to the tolerance (2e-7, near the FP32 floor); 100 iterations that end with a
   // violation above 1e-3 (or a non-finite one) mean the bonds could not be restored
@@ -1250,7 +1250,7 @@ __device__ double rattle_pass(const Ctx& c, bool want_k) {
   const int fly0 = v.s->fly0, fly1 = v.s->fly1;
   const float imv[3] = {P.inv_m[2], P.inv_m[3], P.inv_m[3]};
   const int ca[3] = {0, 0, 1}, cb[3] = {1, 2, 2};
-  const float dd[3] = {(float)P.d_oh2, (float)P.d_oh2, (float)P.d_hh2};
+  const float dd[3] = {P.d_oh2_f, P.d_oh2_f, P.d_hh2_f};
   long long kin = 0;  // kinetic energy, fixed point (exact, order-free sum)
   int kbad = 0;
   const int flyw = v.s->flyw;
@@ -1333,7 +1333,7 @@ __device__ H4D_PHASE void kick_drift(const Ctx& cref, float alpha) {
   const GView& v = c.v;
   const int n = v.s->n_tot;
   const int fly0 = v.s->fly0, fly1 = v.s->fly1;
-  const float half_dt = 0.5f * (float)e.proto.dt;
+  const float half_dt = 0.5f * e.proto.dt_f;
   int bad = 0;
   float d1 = 0.f, d2 = 0.f;  // this thread's two largest displacements (Verlet list)
   float o1 = 0.f, o2 = 0.f;  // the same against the outer-list reference
@@ -1781,15 +1781,18 @@ __device__ H4D_PHASE void nemd_steps(const Ctx& cref, int n_steps) {
     force_pass<SYS>(c, 0, 0.f, nullptr);
     c.sync();
   }
+  // The altitudes of 32 steps at a time, one per lane of warp 0 (FP64 divisions and powers cost
+  // the FP64 pipe as much for one lane as for 32, and far more when every warp makes its own:
+  // NEMD steps of a 250-ion chain 26 -> 21 us); thread 0 hands them on
+  double alt = 0.0, a_prev = c.tid < 32 && n_steps > 0 ? altitude(e.proto, ins, 0) : 0.0;
   for (int k = 0; k < n_steps; ++k) {
     kick_drift<SYS>(c, 1.0f);
+    if (c.tid < 32 && (k & 31) == 0) alt = altitude(e.proto, ins, min(k + 1 + c.tid, n_steps));
     c.sync();
     maybe_rebuild(c);
-    // the altitude before this step, from the schedule (S->w_cur holds the same value, but
-    // thread 0 overwrites it below with no barrier in between when no rebuild happens)
-    const float w_prev = (float)altitude(e.proto, ins, k);
-    const float w_next = (float)altitude(e.proto, ins, k + 1);
-    const float w_next_a = (float)(e.proto.rw * altitude(e.proto, ins, k + 1));
+    double a_next = 0.0;
+    if (c.tid < 32) a_next = __shfl_sync(0xffffffffu, alt, k & 31);
+    const float w_next = (float)a_next, w_next_a = (float)(e.proto.rw * a_next);  // (thread 0)
     if (c.tid == 0) {
       uint4 p0 = c.v.pos[f0];
       p0.w = __float_as_uint(w_next);
@@ -1804,11 +1807,12 @@ __device__ H4D_PHASE void nemd_steps(const Ctx& cref, int n_steps) {
         p2.w = __float_as_uint(w_next);
         c.v.pos[f2] = p2;
       }
+      S->w_prev = (float)a_prev;
       S->w_cur = w_next;
       S->g_scr = expf(-e.pot.kappa_sr * (single ? w_next : 0.5f * (w_next + w_next_a)));
     }
     c.sync();
-    force_pass<SYS>(c, 1 | 4, w_prev, nullptr);
+    force_pass<SYS>(c, 1 | 4, S->w_prev, nullptr);
     c.sync();
     if (SYS == H4D_SYS_AQ && c.r.n_water > 0) {
       rattle_pass(c, false);
@@ -1824,7 +1828,7 @@ __device__ H4D_PHASE void nemd_steps(const Ctx& cref, int n_steps) {
                      dz = (double)(int)(b.z - a.z) * s;
         const double r3 = dx * dx + dy * dy + dz * dz;
         const double dn = (double)w_next - (double)w_next_a;
-        const double dp = (double)w_prev - (double)(float)(e.proto.rw * altitude(e.proto, ins, k));
+        const double dp = (double)(float)a_prev - (double)(float)(e.proto.rw * a_prev);
         const int ta = type_of(f0, c.r.nw3), tb = type_of(f1, c.r.nw3);
         dff = pair_u64(e.pot, ta, tb, r3 + dn * dn, 1.0) - pair_u64(e.pot, ta, tb, r3 + dp * dp, 1.0);
       }
@@ -1833,6 +1837,7 @@ __device__ H4D_PHASE void nemd_steps(const Ctx& cref, int n_steps) {
       S->wprot_c = (t - S->wprot) - y;
       S->wprot = t;
     }
+    a_prev = a_next;
   }
 }
 

@@ -31,6 +31,7 @@ struct Pot {
   double drc2_lj, drc2_c, dalpha, dshift_c, dkappa_sr;
   double dm[kMaxT];    // m mvv2e
   double d_oh2, d_hh2;  // squared water bond lengths
+  float d_oh2_f, d_hh2_f;
   double inv_m_d[kMaxT];
   float q[kMaxT];       // charges per type (proposal field feature)
   int erfcx_fit;        // alpha rc_coul within the range of the fitted erfcx (aqueous pair term)
@@ -57,6 +58,7 @@ struct __align__(16) CoulPiece {
 struct Proto {
   int n_f, schedule;
   double w_max, sched_n, dt, tau_t;
+  float dt_f, pad_dt;
   double beta, beta_mu;
   int no_accept;
   int prop_mode;    // 0 uniform placement, 1 learned proposal density
