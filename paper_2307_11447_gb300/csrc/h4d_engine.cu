@@ -45,6 +45,11 @@ __device__ __forceinline__ void gsync(int bar, int nthreads) {
 __device__ __forceinline__ int type_of(int a, int nw3) {
   return a < nw3 ? ((a % 3 == 0) ? 2 : 3) : ((a - nw3) & 1);
 }
+// the same without a division: multiples of 3 are those that its inverse mod 2^32 maps below 2^32 / 3
+__device__ __forceinline__ unsigned type_of_u(unsigned a, int nw3) {
+  const unsigned water = a * 0xAAAAAAABu <= 0x55555555u ? 2u : 3u;
+  return (int)a < nw3 ? water : ((a - (unsigned)nw3) & 1u);
+}
 template <int SYS>
 __device__ __forceinline__ int type_t(int a, int nw3) {
   if (SYS == H4D_SYS_LJ) return a & 1;  // no waters: ions alternate cation/anion
@@ -93,11 +98,17 @@ __device__ __forceinline__ float as_erfc_poly(float x) {
   p = fmaf(t, p, 0.254829592f);
   return p * t;
 }
+// 1/d for d in [1, 3]: the approximation and one Newton step
+__device__ __forceinline__ float recip_near1(float d) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return fmaf(r, fmaf(-d, r, 1.0f), r);
+}
 // erfcx(x) = e^{x^2} erfc(x) on [0, 3.2] as t sum_k c_k t^k, t = 1/(1 + x/2), with the
 // coefficients printed by fit_erfcx.py (a least-squares fit in relative error, reweighted
 // toward minimax: 1.3e-10 in exact arithmetic, 3.3e-7 in this float32 evaluation)
 __device__ __forceinline__ float erfcx_poly(float x) {
-  const float t = __frcp_rn(fmaf(0.5f, x, 1.0f));
+  const float t = recip_near1(fmaf(0.5f, x, 1.0f));
   float p = 3.845890611e-02f;
   p = fmaf(p, t, -2.708916664e-01f);
   p = fmaf(p, t, 7.915914059e-01f);
@@ -231,6 +242,38 @@ __device__ __forceinline__ void pair_fr_lj2_poly(const Pot& P, float2 r2, float2
   fr_c = __fmul2_rn(kqg, __ffma2_rn(rinv2, rinv, cp));
 }
 
+// Two aqueous pair terms at once: the operations of pair_fr<H4D_SYS_AQ> in the same order, each
+// half rounded like its scalar counterpart.  t: sigma^2, 4 epsilon and charge product of each
+// pair; kqg: the charge products times their screening factors.  FIT: erfc from the fitted erfcx.
+template <bool FIT>
+__device__ __forceinline__ float2 pair_fr_aq2(const Pot& P, float2 r2, float2 sig2, float2 eps4, float2 kqg) {
+  const float2 rinv = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
+  const float2 rinv2 = __fmul2_rn(rinv, rinv);
+  const float2 s2 = __fmul2_rn(sig2, rinv2);
+  const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
+  const float2 lj = __fmul2_rn(__fmul2_rn(__fmul2_rn(eps4, s6), __ffma2_rn(f2(12.0f), s6, f2(-6.0f))), rinv2);
+  const float2 x = __fmul2_rn(f2(P.alpha), __fmul2_rn(r2, rinv));
+  const float2 y = __fmul2_rn(__fmul2_rn(make_float2(-x.x, -x.y), x), f2(1.4426950408889634f));
+  const float2 ex = make_float2(ex2_approx(y.x), ex2_approx(y.y));
+  float2 erfcx;
+  if (FIT) {
+    const float2 d = __ffma2_rn(f2(0.5f), x, f2(1.0f));
+    const float2 r0 = make_float2(rcp_approx(d.x), rcp_approx(d.y));
+    const float2 t = __ffma2_rn(r0, __ffma2_rn(make_float2(-d.x, -d.y), r0, f2(1.0f)), r0);
+    constexpr float c[10] = {2.818836868e-01f, 2.859359086e-01f,  2.157940567e-01f, 3.224146068e-01f,  -3.565987349e-01f,
+                             8.702221513e-01f, -1.178810358e+00f, 7.915914059e-01f, -2.708916664e-01f, 3.845890611e-02f};
+    float2 p = f2(c[9]);
+#pragma unroll
+    for (int k = 8; k >= 0; --k) p = __ffma2_rn(p, t, f2(c[k]));
+    erfcx = __fmul2_rn(ex, __fmul2_rn(p, t));
+  } else {
+    erfcx = make_float2(erfcf(x.x), erfcf(x.y));
+  }
+  const float2 co = __fmul2_rn(__fmul2_rn(kqg, __ffma2_rn(erfcx, rinv, __fmul2_rn(f2(P.two_alpha_sqrtpi), ex))), rinv2);
+  return make_float2((r2.x < P.rc2_lj ? lj.x : 0.0f) + (r2.x < P.rc2_c ? co.x : 0.0f),
+                     (r2.y < P.rc2_lj ? lj.y : 0.0f) + (r2.y < P.rc2_c ? co.y : 0.0f));
+}
+
 // FP32 pair energy (protocol-work diagnostic only)
 template <int SYS>
 __device__ __forceinline__ float pair_u32(const Pot& P, const PairCoef<SYS>& c, float r2, float g) {
@@ -284,13 +327,15 @@ struct GScal {
   unsigned int xfly[6];
   double vw[9];            // velocities of an inserted water (O, H, H)
   unsigned int xw[9];      // its fixed-point coordinates
-  double kw[32];
+  union {  // scratch of the group's reductions, between barriers
+    double kw[32];
+    float pmw[2][32];      // per-warp maxima of the proposal logits
+  };
   float d1w[32], d2w[32];  // per-warp largest and second-largest displacement since the build
   float o1w[32], o2w[32];  // the same since the outer-list build
   int next_item, n_items;  // dynamic work items of the outer build
   // learned proposal of the current trial
   float pm[2];             // largest cation / anion logit
-  float pmw[2][32];        // per-warp maxima
   double pZ[2];            // softmax normalisers sum_k exp(l_k - max)
   double lnq;              // log proposal factor of the trial
   int cell_c, cell_a;      // grid cells of the exchanged cation and anion
@@ -298,6 +343,8 @@ struct GScal {
   int n_rank;              // atoms ranked in lrank for the next outer build (0 = none)
   int n_lay;               // atoms of the outer-row layout in lord (0 = rows by index)
   int pad_l;
+  // aqueous pair constants per (ti * 4 + tj): sigma^2, 4 epsilon, charge product
+  alignas(16) float4 pt[16];
 };
 static_assert(sizeof(GScal) <= 1536, "per-group scalars exceed their shared-memory slot");
 
@@ -1001,6 +1048,61 @@ __device__ __forceinline__ void lj_row(const Pot& P, const uint4* __restrict__ p
   }
 }
 
+// One atom's aqueous row on this lane, four slots per packet, two pair terms at a time.  The
+// per-atom force is a sum of hundreds of large, cancelling Coulomb terms, so it is accumulated
+// with Kahan compensation (cx, cy, cz).  The pair constants come from a table in shared memory
+// (tab: the row of the atom's type; indexed constant loads are replayed for every distinct pair
+// of types in a warp), and the sentinel's infinite altitude puts padding beyond every cut-off.
+// Bound: issue slots (a warp issues in 55% of the cycles) with the FP32 and ALU pipes and the
+// position gathers each about half busy.  Force pass of 152 chains of 9110 atoms 2.19 -> 1.83 ms,
+// of 1370 atoms 0.355 -> 0.277 ms; selecting the constants by type in registers 1.87 ms.
+template <bool NEMD, bool FIT>
+__device__ __forceinline__ void aq_row(const Pot& P, const uint4* __restrict__ pos, const float4* __restrict__ tab,
+                                       const uint2* pk, size_t pstride, int npk, uint2 q, int nw3, const uint4& pi,
+                                       float scale, float wi, bool wnz_i, float gscr, float& fx, float& fy, float& fz,
+                                       float& cx, float& cy, float& cz) {
+  for (int p = 0; p < npk; ++p) {
+    uint2 qn = make_uint2(0u, 0u);
+    if (p + 1 < npk) qn = ld_packet(pk + (size_t)(p + 1) * pstride);
+    if (H4D_PF_FORCE > 0 && p + H4D_PF_FORCE < npk) prefetch_l2(pk + (size_t)(p + H4D_PF_FORCE) * pstride);
+    const unsigned jw[4] = {q.x & 0xFFFFu, q.x >> 16, q.y & 0xFFFFu, q.y >> 16};
+#pragma unroll
+    for (int h = 0; h < 4; h += 2) {
+      const uint4 pa = pos[jw[h]], pb = pos[jw[h + 1]];
+      const float4 ta = tab[type_of_u(jw[h], nw3)], tb = tab[type_of_u(jw[h + 1], nw3)];
+      const float2 dx = __fmul2_rn(make_float2((float)(int)(pa.x - pi.x), (float)(int)(pb.x - pi.x)), f2(scale));
+      const float2 dy = __fmul2_rn(make_float2((float)(int)(pa.y - pi.y), (float)(int)(pb.y - pi.y)), f2(scale));
+      const float2 dz = __fmul2_rn(make_float2((float)(int)(pa.z - pi.z), (float)(int)(pb.z - pi.z)), f2(scale));
+      float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+      const float2 wj = make_float2(wbits(pa), wbits(pb));  // 0, a flyer's altitude, or +inf
+      float2 kqg = make_float2(ta.z, tb.z);
+      if (NEMD) {
+        const float2 dw = __fadd2_rn(f2(wi), make_float2(-wj.x, -wj.y));
+        r2 = __ffma2_rn(dw, dw, r2);
+        kqg.x = (wnz_i != (wj.x != 0.0f)) ? kqg.x * gscr : kqg.x;
+        kqg.y = (wnz_i != (wj.y != 0.0f)) ? kqg.y * gscr : kqg.y;
+      } else {
+        r2 = __ffma2_rn(wj, wj, r2);
+      }
+      const float2 fr = pair_fr_aq2<FIT>(P, r2, make_float2(ta.x, tb.x), make_float2(ta.y, tb.y), kqg);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {  // in slot order
+        const float f = k ? fr.y : fr.x;
+        const float tx = fmaf(-f, k ? dx.y : dx.x, -cx), ty = fmaf(-f, k ? dy.y : dy.x, -cy),
+                    tz = fmaf(-f, k ? dz.y : dz.x, -cz);
+        const float sx = fx + tx, sy = fy + ty, sz = fz + tz;
+        cx = (sx - fx) - tx;
+        cy = (sy - fy) - ty;
+        cz = (sz - fz) - tz;
+        fx = sx;
+        fy = sy;
+        fz = sz;
+      }
+    }
+    q = qn;
+  }
+}
+
 // ------------------------------------------------------------------------------------
 // Force pass (FP32): tpa lanes per atom over its full row, butterfly reduction.
 // mode bits: 1 = apply the second half kick, 2 = accumulate kinetic partials,
@@ -1069,49 +1171,12 @@ __device__ H4D_PHASE void force_pass_impl(const Ctx& cref, int mode, float w_pre
           lj_row<NEMD, 2>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
         else
           lj_row<NEMD, 0>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
-      } else
-      for (int p = 0; p < npk; ++p) {
-        uint2 qn = make_uint2(0u, 0u);
-        if (p + 1 < npk) qn = ld_packet(pk + (size_t)(p + 1) * pstride);
-        const int jj[4] = {(int)(q.x & 0xFFFFu), (int)(q.x >> 16), (int)(q.y & 0xFFFFu), (int)(q.y >> 16)};
-        // branch-free over the four slots: a padding slot (the sentinel) gets r^2 = 1e30, for
-        // which every term of the pair function is exactly zero
-        uint4 pj[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) pj[u] = v.pos[jj[u]];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const bool valid = jj[u] != R.cap_atoms;
-          const float dx = (float)(int)(pj[u].x - pi.x) * scale;
-          const float dy = (float)(int)(pj[u].y - pi.y) * scale;
-          const float dz = (float)(int)(pj[u].z - pi.z) * scale;
-          float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          float g = 1.0f;
-          if (NEMD) {
-            const float wj = wbits(pj[u]);
-            const float dw = wi - wj;
-            r2 = fmaf(dw, dw, r2);
-            g = (wnz_i != (wj != 0.0f)) ? gscr : 1.0f;
-          }
-          r2 = valid ? r2 : 1.0e30f;
-          const PairCoef<SYS> cf = coef<SYS>(P, ti, type_t<SYS>(jj[u] & 0x7FFF, R.nw3));
-          const float fr = pair_fr<SYS>(P, cf, r2, g);
-          if (SYS == H4D_SYS_AQ) {
-            const float tx = -fr * dx - cx, ty = -fr * dy - cy, tz = -fr * dz - cz;
-            const float sx = fx + tx, sy = fy + ty, sz = fz + tz;
-            cx = (sx - fx) - tx;
-            cy = (sy - fy) - ty;
-            cz = (sz - fz) - tz;
-            fx = sx;
-            fy = sy;
-            fz = sz;
-          } else {
-            fx = fmaf(-fr, dx, fx);
-            fy = fmaf(-fr, dy, fy);
-            fz = fmaf(-fr, dz, fz);
-          }
-        }
-        q = qn;
+      } else if (P.erfcx_fit) {
+        aq_row<NEMD, true>(P, v.pos, v.s->pt + 4 * ti, pk, pstride, npk, q, R.nw3, pi, scale, wi, wnz_i, gscr, fx, fy,
+                           fz, cx, cy, cz);
+      } else {
+        aq_row<NEMD, false>(P, v.pos, v.s->pt + 4 * ti, pk, pstride, npk, q, R.nw3, pi, scale, wi, wnz_i, gscr, fx, fy,
+                            fz, cx, cy, cz);
       }
       if (NEMD && (mode & 4) && iflyer) {
         // protocol work of a flying row: U(w_now) - U(w_prev) against every non-flyer
@@ -2813,6 +2878,7 @@ __device__ bool setup_ctx(const Eng& e, char* smem, Ctx& c) {
     S->w_cur = 0.f; S->g_scr = 1.f;
     write_sentinel(c.v, R->cap_atoms);
   }
+  if (c.tid < 16) S->pt[c.tid] = make_float4(e.pot.sig2[c.tid], e.pot.eps4[c.tid], e.pot.kq[c.tid], 0.f);
   c.sync();
   for (int a = c.tid; a < S->n_tot; a += c.T) c.v.pos[a] = e.pos[R->atom_off + a];
   c.sync();
@@ -2943,6 +3009,7 @@ __global__ void __launch_bounds__(1024) eval_kernel(const __grid_constant__ Eng 
     S->g_scr = expf(-e.pot.kappa_sr * wbar);
     write_sentinel(c.v, R->cap_atoms);
   }
+  if (c.tid < 16) S->pt[c.tid] = make_float4(e.pot.sig2[c.tid], e.pot.eps4[c.tid], e.pot.kq[c.tid], 0.f);
   c.sync();
   for (int a = c.tid; a < S->n_tot; a += c.T) c.v.pos[a] = e.pos[R->atom_off + a];
   c.sync();
