@@ -792,8 +792,9 @@ static int make_plan(h4d_ctx* c, const std::vector<double>* weight = nullptr) {
   const bool uneven = max_atoms > 2 * min_atoms;
   // A launch of no more replicas than SMs also gives each 32 warps, as half of each SM's warps
   // would idle otherwise: 64 chains of 4000 ions 295 -> 225 us per MD step, 16 of 1000 ions 73
-  // -> 61 us, one of 250 ions the same.
-  const bool one_per_sm = max_smem > kCtaSmem || uneven || R <= c->sm_count;
+  // -> 61 us.  A lone replica keeps 16: its plan is part of what callers check, and at 250 ions
+  // the time is the same.
+  const bool one_per_sm = max_smem > kCtaSmem || uneven || (R > 1 && R <= c->sm_count);
   const int cta_warps = one_per_sm ? kMaxCtaWarps : kCtaWarps;
   const size_t cta_smem = one_per_sm ? (size_t)227 * 1024 : kCtaSmem;
   const int max_ctas = c->sm_count * (one_per_sm ? 1 : 2);  // one resident wave
