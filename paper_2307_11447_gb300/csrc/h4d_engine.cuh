@@ -90,7 +90,7 @@ struct Rep {
   int nc;         // cells per dimension (0 = all pairs)
   int reach;      // stencil half-width: cells are at least r_list / reach wide
   int tpa;
-  int pad_r;
+  int lanes;      // lanes of a warp that share a row: tpa, or fewer, each taking several of its parts (0: tpa)
   unsigned long long T_list;   // neighbour criterion threshold (fixed-point units^2)
   unsigned long long T_move;   // (skin/2)^2 in fixed-point units^2
   float skin_fx;               // skin in fixed-point units
