@@ -344,7 +344,7 @@ class Context:
         v = np.empty((cap, 3))
         n = ctypes.c_int64()
         _ck(lib().h4d_get_state(self.h, r, _pd(x), _pd(v), cap, ctypes.byref(n)), "h4d_get_state")
-        return x[: n.value].copy(), v[: n.value].copy()
+        return x[: n.value], v[: n.value]
 
     def h4d_set_state(self, r, n_pairs, x, v):
         x = np.ascontiguousarray(x, np.float64)
