@@ -119,21 +119,32 @@ __global__ void __launch_bounds__(32 * kSkWarps, 2)
   // plane, lane and half of this lane's column in At
   float* const Aw = At + ((lane & 2) >> 1) * 32 + (lane >> 2) * 4 + (lane & 1) * 2;
   for (int t0 = a0; t0 < a1; t0 += kStage) {
-    __syncthreads();
-#pragma unroll 2
-    for (int a = warp; a < kStage; a += kSkWarps) {
-      const uint4 p = t0 + a < a1 ? xq[t0 + a] : make_uint4(0u, 0u, 0u, 0u);
-      const float q = __uint_as_float(p.w);
-      float c, s;
-      phase_cs((unsigned)mycol.x * p.x + (unsigned)mycol.y * p.y, c, s);
-      *reinterpret_cast<float2*>(Aw + a * 64) = make_float2(q * c, q * s);
+    // (all of the stage's loads ahead of its arithmetic: one wait for L2 instead of four)
+    uint4 p[kStage / kSkWarps];
+    unsigned z[kStage * kMT / (32 * kSkWarps)];
+#pragma unroll
+    for (int r = 0; r < kStage / kSkWarps; ++r) {
+      const int a = t0 + warp + r * kSkWarps;
+      p[r] = a < a1 ? xq[a] : make_uint4(0u, 0u, 0u, 0u);
     }
-#pragma unroll 2
-    for (int e = threadIdx.x; e < kStage * kMT; e += 32 * kSkWarps) {
-      const int a = e / kMT, m = e % kMT;
-      const unsigned z = t0 + a < a1 ? xq[t0 + a].z : 0u;
+#pragma unroll
+    for (int r = 0; r < kStage * kMT / (32 * kSkWarps); ++r) {
+      const int a = t0 + threadIdx.x / kMT + r * (32 * kSkWarps / kMT);
+      z[r] = a < a1 ? xq[a].z : 0u;
+    }
+    __syncthreads();  // the tables of the stage before are done with
+#pragma unroll
+    for (int r = 0; r < kStage / kSkWarps; ++r) {
+      const float q = __uint_as_float(p[r].w);
       float c, s;
-      phase_cs((unsigned)(mt * kMT + m) * z, c, s);
+      phase_cs((unsigned)mycol.x * p[r].x + (unsigned)mycol.y * p[r].y, c, s);
+      *reinterpret_cast<float2*>(Aw + (warp + r * kSkWarps) * 64) = make_float2(q * c, q * s);
+    }
+#pragma unroll
+    for (int r = 0; r < kStage * kMT / (32 * kSkWarps); ++r) {
+      const int a = threadIdx.x / kMT + r * (32 * kSkWarps / kMT), m = threadIdx.x % kMT;
+      float c, s;
+      phase_cs((unsigned)(mt * kMT + m) * z[r], c, s);
       *reinterpret_cast<float4*>(Bt + a * 64 + 4 * m) = make_float4(c, c, s, s);
     }
     __syncthreads();
