@@ -13,7 +13,7 @@
 // theirs.  Both passes are then small matrix products: the structure factors contract
 // columns x n_z over the atoms, the forces contract columns x atoms over n_z.  Bound: the FP32
 // pipe and, at about a quarter of the instructions, the sines and cosines of the tables.  A call for 9110
-// atoms at kmax 14 with forces: 993 -> 322 us, of which the two passes take 32 us each (one
+// atoms at kmax 14 with forces: 993 -> 156 us, of which the kernels take 78 us (one
 // sincospif per term, the k-space weights on the host and a copy each way between the passes took
 // 330 us of kernels); error of the forces against 64 bits 6.3e-6 -> 1.9e-6.
 #include <cuda_runtime.h>
@@ -25,7 +25,7 @@
 #include <new>
 #include <vector>
 
-#include "../../include/h4d.h"
+#include "h4d_engine.cuh"
 
 namespace {
 
@@ -379,8 +379,9 @@ extern "C" int h4d_ewald_lr(const h4d_params* params, double L, int32_t n_water,
   } catch (const std::bad_alloc&) {
     return H4D_ECUDA;
   }
-  unsigned char* b = nullptr;
-  if (cudaMalloc(&b, off) != cudaSuccess) return H4D_ECUDA;
+  void* slab = nullptr;
+  if (h4d::scratch_alloc(&slab, off) != H4D_OK) return H4D_ECUDA;
+  unsigned char* b = static_cast<unsigned char*>(slab);
   uint4* xq = reinterpret_cast<uint4*>(b + o_xq);
   double* d_x = reinterpret_cast<double*>(b + o_x);
   double* d_u = reinterpret_cast<double*>(b + o_u);
@@ -425,9 +426,10 @@ extern "C" int h4d_ewald_lr(const h4d_params* params, double L, int32_t n_water,
     good = ok(cudaEventElapsedTime(&ms, ev[0], ev[1]));
     *t_kernel_ms = ms;
   }
+  if (!good) cudaStreamSynchronize(0);
   for (auto& e : ev)
     if (e) cudaEventDestroy(e);
-  cudaFree(b);
+  h4d::scratch_free(b);
   if (!good) return H4D_ECUDA;
   double sum = 0.0;
   for (int k = 0; k < n_u; ++k) sum += u[k];
