@@ -850,6 +850,15 @@ int scratch_alloc(void** p, size_t bytes) {
 }
 
 void scratch_free(void* p) { cudaFreeAsync(p, 0); }
+
+// what the pool of the current device still keeps goes back to the device
+static void scratch_trim() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  const auto it = g_pools.find(dev);
+  if (it != g_pools.end()) cudaMemPoolTrimTo(it->second, 0);
+}
 }  // namespace h4d
 
 static int check_device() {
@@ -1081,6 +1090,7 @@ void h4d_destroy(h4d_ctx* c) {
   if (c->pin) cudaFreeHost(c->pin);
   invalidate_graphs(c);
   if (c->own_stream) cudaStreamDestroy(c->stream);
+  scratch_trim();
   delete c;
 }
 
