@@ -169,7 +169,9 @@ struct h4d_ctx {
   h4d_record* d_rec = nullptr;
   double* d_scratch = nullptr;
   unsigned long long* d_count = nullptr;
-  // pinned staging of the getters (grown on demand, kept with the context)
+  // pinned staging of the getters (grown on demand, kept with the context).  pin_mu is held from
+  // staging() until the result has been copied out: several threads may read one context
+  std::mutex pin_mu;
   unsigned char* pin = nullptr;
   size_t pin_bytes = 0;
   // learned proposal: network (FP32 masters, Adam moments, packed bf16 fragments), grid,
@@ -606,7 +608,7 @@ static int pull_reps(h4d_ctx* c) {
   return H4D_OK;
 }
 
-// Pinned staging of at least `bytes`; pageable copies make the driver stage and wait once
+// Pinned staging of at least `bytes` (under pin_mu); pageable copies make the driver stage and wait once
 // each (85 us per state of 4000 ions).
 static unsigned char* staging(h4d_ctx* c, size_t bytes) {
   if (bytes > c->pin_bytes) {
@@ -1262,6 +1264,7 @@ int h4d_autotune(h4d_ctx* c, int32_t n_iter, double* pass_ns, double* build_ns) 
 
 int h4d_get_counts(h4d_ctx* c, int32_t r, h4d_counts* out) {
   if (!c || !out || r < 0 || r >= c->R) return H4D_EINVAL;
+  const std::lock_guard<std::mutex> lock(c->pin_mu);
   int rc = pull_rep(c, r);
   if (rc) return rc;
   const Rep& R = c->rep_h[r];
@@ -1315,6 +1318,7 @@ int h4d_get_energies(h4d_ctx* c, int32_t r, double* U, double* K) {
 
 int h4d_get_work(h4d_ctx* c, int32_t r, h4d_record* out, int64_t cap, int64_t* n) {
   if (!c || r < 0 || r >= c->R || (cap > 0 && !out)) return H4D_EINVAL;
+  const std::lock_guard<std::mutex> lock(c->pin_mu);
   const int64_t most = std::max<int64_t>(0, std::min<int64_t>(cap, c->rep_h[r].rec_cap));
   std::vector<unsigned char> own;
   const unsigned char* p = nullptr;
@@ -1332,6 +1336,7 @@ int h4d_get_work(h4d_ctx* c, int32_t r, h4d_record* out, int64_t cap, int64_t* n
 
 int h4d_get_state(h4d_ctx* c, int32_t r, double* x, double* v, int64_t cap_atoms, int64_t* n_atoms) {
   if (!c || r < 0 || r >= c->R) return H4D_EINVAL;
+  const std::lock_guard<std::mutex> lock(c->pin_mu);
   const size_t cap = (size_t)c->rep_h[r].cap_atoms, block = cap * 3 * sizeof(double);
   const size_t o_v = kExportHead + (x ? block : 0);
   std::vector<unsigned char> own;

@@ -1,0 +1,65 @@
+"""The host side of libh4d over a CUDA runtime that needs no GPU (tests/host/fake_cudart.c,
+preloaded in a child process): what several threads, several devices and failing calls do to it."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+from paper_2307_11447_gb300 import lib as h4d
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SETUP = """
+import ctypes, sys
+import numpy as np
+from concurrent.futures import ThreadPoolExecutor
+from paper_2307_11447_gb300 import lib as h4d, workloads as wl
+rt = ctypes.CDLL(None)
+cfg = wl.lj_config(100, 0.1, 10)
+
+def context(R):
+    rng = np.random.default_rng(1)
+    reps = [dict(L=cfg["L"], n_pairs=50 - r, cap_pairs=60, x=rng.uniform(0, cfg["L"], (100 - 2 * r, 3)),
+                 v=rng.normal(size=(100 - 2 * r, 3))) for r in range(R)]
+    return h4d.Context(h4d.make_params(cfg), reps, seed=1), reps
+"""
+
+
+@pytest.fixture(scope="session")
+def runtime(tmp_path_factory):
+    h4d.lib()  # built before the children load it
+    out = tmp_path_factory.mktemp("host") / "fake_cudart.so"
+    inc = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    subprocess.check_call(["gcc", "-O1", "-Wall", "-fPIC", "-shared", "-I", inc, "-o", str(out),
+                           os.path.join(ROOT, "tests", "host", "fake_cudart.c")])
+
+    def run(code):
+        env = dict(os.environ, LD_PRELOAD=str(out), PYTHONPATH=ROOT)
+        r = subprocess.run([sys.executable, "-c", SETUP + code], env=env, cwd=ROOT, capture_output=True, text=True, timeout=120)
+        assert r.returncode == 0 and r.stdout.endswith("ok\n"), (r.returncode, r.stdout, r.stderr)
+
+    return run
+
+
+def test_getters_from_several_threads_read_what_one_thread_reads(runtime):
+    runtime("""
+ctx, reps = context(8)
+want = [ctx.h4d_get_state(r) for r in range(8)]
+for r, rep in enumerate(reps):
+    assert np.abs(want[r][0] - rep["x"]).max() < 1e-8 and np.abs(want[r][1] - rep["v"]).max() < 1e-6
+
+def read(t):
+    bad = 0
+    for k in range(60):
+        r = (t + k) % 8
+        x, v = ctx.h4d_get_state(r)
+        bad += not (np.array_equal(x, want[r][0]) and np.array_equal(v, want[r][1]))
+        bad += ctx.h4d_get_counts(r)["n_pairs"] != 50 - r
+    return bad
+
+with ThreadPoolExecutor(8) as ex:
+    bad = sum(ex.map(read, range(8)))
+assert bad == 0, bad
+ctx.close()
+print("ok")
+""")
