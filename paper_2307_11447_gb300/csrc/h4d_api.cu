@@ -140,6 +140,7 @@ struct h4d_ctx {
   int cta_threads;
   int n_ctas;
   size_t smem;
+  int device = 0;  // current when the context was created: its memory and streams are there
   std::vector<Rep> rep_h;
   std::vector<Group> groups_h;
   std::vector<int> cta_groups_h;
@@ -608,6 +609,19 @@ static int pull_reps(h4d_ctx* c) {
   return H4D_OK;
 }
 
+// The context's device as the current one while a getter launches on its stream (a launch, unlike
+// a copy, is refused when another device is current)
+struct OnDevice {
+  int back = -1;
+  explicit OnDevice(int device) {
+    int now = 0;
+    if (cudaGetDevice(&now) == cudaSuccess && now != device && cudaSetDevice(device) == cudaSuccess) back = now;
+  }
+  ~OnDevice() {
+    if (back >= 0) cudaSetDevice(back);
+  }
+};
+
 // Pinned staging of at least `bytes` (under pin_mu); pageable copies make the driver stage and wait once
 // each (85 us per state of 4000 ions).
 static unsigned char* staging(h4d_ctx* c, size_t bytes) {
@@ -628,6 +642,7 @@ static unsigned char* staging(h4d_ctx* c, size_t bytes) {
 
 // one replica's table entry (the getters of one replica need no other)
 static int pull_rep(h4d_ctx* c, int r) {
+  const OnDevice on(c->device);
   Rep* p = reinterpret_cast<Rep*>(staging(c, sizeof(Rep)));
   if (!p) return pull_reps(c);
   CK(cudaMemcpyAsync(p, c->d_rep + r, sizeof(Rep), cudaMemcpyDeviceToHost, c->stream));
@@ -686,6 +701,7 @@ static __global__ void __launch_bounds__(256) export_records(const Rep* __restri
 // pinned memory, in `own` by way of a device buffer
 template <class Launch>
 static int export_to_host(h4d_ctx* c, size_t bytes, std::vector<unsigned char>& own, const unsigned char** p, Launch launch) {
+  const OnDevice on(c->device);
   if (unsigned char* pin = staging(c, bytes)) {
     launch(pin);
     CK(cudaGetLastError());
@@ -1029,6 +1045,7 @@ int h4d_create(const h4d_params* params, const h4d_system* sys, uint64_t seed, v
     cudaDeviceProp prop;
     if (cudaGetDevice(&dev) == cudaSuccess && cudaGetDeviceProperties(&prop, dev) == cudaSuccess)
       c->sm_count = prop.multiProcessorCount;
+    c->device = dev;
   }
   c->R = sys->n_replicas;
   c->max_nbr = params->max_nbr > 0 ? params->max_nbr : derive_max_nbr(*params);

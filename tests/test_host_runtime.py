@@ -63,3 +63,19 @@ assert bad == 0, bad
 ctx.close()
 print("ok")
 """)
+
+
+def test_getters_work_from_another_current_device(runtime):
+    runtime("""
+ctx, reps = context(2)
+x0, v0 = ctx.h4d_get_state(1)
+c0 = ctx.h4d_get_counts(1)
+rt.cudaSetDevice(1)
+x1, v1 = ctx.h4d_get_state(1)
+assert np.array_equal(x0, x1) and np.array_equal(v0, v1)
+assert len(ctx.h4d_get_work(1, 4)) == 0 and ctx.h4d_get_counts(1) == c0
+dev = ctypes.c_int(-1)
+rt.cudaGetDevice(ctypes.byref(dev))
+assert dev.value == 1
+print("ok")
+""")
