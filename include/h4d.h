@@ -28,7 +28,10 @@
  *     exception crosses the ABI.  h4d_strerror() names each code.
  *   - Pointers named host_* are host memory; the library copies from or into them and
  *     never keeps them.  Pointers named dev_* are device memory owned by the caller.
- *     All other device memory is owned by the context and freed by h4d_destroy().
+ *     All other device memory is owned by the context and freed by h4d_destroy(), except
+ *     for scratch of the stateless calls: up to 16 MiB of it per device stay with the library
+ *     between calls (after calls of several threads, up to what they used at once, until the
+ *     next wait on the device); h4d_destroy() of any context gives it back.
  *   - Each context issues its work on the CUDA stream given at creation; with NULL the
  *     context creates a non-blocking stream of its own (CUDA-graph capture cannot use
  *     the legacy default stream) and destroys it in h4d_destroy().  Launching entry

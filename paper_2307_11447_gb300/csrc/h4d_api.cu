@@ -834,7 +834,9 @@ static int upload_replica(h4d_ctx* c, int r, int n_pairs, const double* x, const
 namespace h4d {
 // One pool per device, made on first use.  cudaMalloc and cudaFree of a call's buffers took 40 and
 // 32 us, a tenth of these calls and more; the pool hands memory out in stream order, so calls
-// from several threads are safe, and returns all above kScratchKeep at the next wait.  Calls of
+// from several threads are safe.  It keeps what is freed to it, up to kScratchKeep, and gives more
+// back only at the next wait, which a call does not make after its last free: a call that needs
+// more than kScratchKeep allocates and frees its own.  Calls of
 // h4d_eval_forces (1000 ions) 300 -> 145 us, h4d_ewald_lr (9110 atoms) 316 -> 150 us,
 // h4d_proposal_grad (4096 records; fifteen allocations before) 490 -> 106 us, the device query of
 // check_device included.
@@ -842,6 +844,7 @@ static std::mutex g_pool_mu;
 static std::map<int, cudaMemPool_t> g_pools;
 
 int scratch_alloc(void** p, size_t bytes) {
+  if (bytes > kScratchKeep) return cudaMalloc(p, bytes) == cudaSuccess ? H4D_OK : H4D_ECUDA;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return H4D_ECUDA;
   cudaMemPool_t pool = nullptr;
@@ -867,7 +870,10 @@ int scratch_alloc(void** p, size_t bytes) {
   return cudaMallocFromPoolAsync(p, bytes, pool, 0) == cudaSuccess ? H4D_OK : H4D_ECUDA;
 }
 
-void scratch_free(void* p) { cudaFreeAsync(p, 0); }
+void scratch_free(void* p, size_t bytes) {
+  if (bytes > kScratchKeep) cudaFree(p);
+  else cudaFreeAsync(p, 0);
+}
 
 // what the pool of the current device still keeps goes back to the device
 static void scratch_trim() {
@@ -1871,7 +1877,7 @@ extern "C" int h4d_eval_forces(const h4d_params* params, double L, int32_t n_wat
   }
   good = good && ok(cudaMemcpy(res.data(), out, n_out * sizeof(double), cudaMemcpyDeviceToHost));
   if (!good) cudaStreamSynchronize(0);
-  scratch_free(b);
+  scratch_free(b, off);
   if (!good) return H4D_ECUDA;
   if (res[0] != 0.0) return eval_forces_lists(params, L, n_water, n, x, w, F, U);
   double u = 0.0, comp = 0.0;
@@ -2281,7 +2287,7 @@ int h4d_proposal_grad(const double* w, int64_t n_rec, const float* feat, const f
   if (!rc) rc = prop_loss_grad(&D, n, s);
   struct { double l; float g[kPropNW]; } out;
   if (cudaMemcpy(&out, D.loss, sizeof(double) + sizeof(out.g), cudaMemcpyDeviceToHost) != cudaSuccess) rc = H4D_ECUDA;
-  scratch_free(slab);
+  scratch_free(slab, off);
   if (!rc) {
     if (loss) *loss = out.l / n;
     if (grad)

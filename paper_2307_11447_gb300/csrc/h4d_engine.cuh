@@ -183,10 +183,10 @@ int point_plan(int n, int* warps, int* homes, int* ctas);  // returns the number
 int launch_point(const Point& a, int warps, int ctas, void* stream);
 
 // Device scratch of one stateless call on the default stream (h4d_api.cu): from a memory pool that
-// keeps at most kScratchKeep bytes between calls
+// keeps at most kScratchKeep bytes between calls; more than that is allocated and freed by the call
 constexpr size_t kScratchKeep = (size_t)16 << 20;
 int scratch_alloc(void** p, size_t bytes);
-void scratch_free(void* p);  // the call's work has been waited for, or it failed
+void scratch_free(void* p, size_t bytes);  // the call's work has been waited for, or it failed
 
 // shared-memory bytes a group needs for a replica
 __host__ __device__ inline size_t smem_align16(size_t b) { return (b + 15) & ~(size_t)15; }

@@ -429,7 +429,7 @@ extern "C" int h4d_ewald_lr(const h4d_params* params, double L, int32_t n_water,
   if (!good) cudaStreamSynchronize(0);
   for (auto& e : ev)
     if (e) cudaEventDestroy(e);
-  h4d::scratch_free(b);
+  h4d::scratch_free(b, off);
   if (!good) return H4D_ECUDA;
   double sum = 0.0;
   for (int k = 0; k < n_u; ++k) sum += u[k];

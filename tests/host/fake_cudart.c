@@ -20,9 +20,33 @@ static cudaError_t ret(cudaError_t e) {
   if (e != cudaSuccess) t_last = e;
   return e;
 }
-static cudaError_t give(void **p, size_t n) {
-  *p = calloc(1, n ? n : 1);
-  return ret(*p ? cudaSuccess : cudaErrorMemoryAllocation);
+static size_t held;
+struct pool { size_t idle; unsigned long long keep; };
+struct head { size_t n; struct pool *from; char fill[240]; };
+static struct pool *pools[16];
+static int n_pools;
+size_t fake_device_bytes(void) { return held; }
+static cudaError_t give(void **p, size_t n, struct pool *from) {
+  struct head *h = calloc(1, sizeof *h + n);
+  if (!h) return ret(cudaErrorMemoryAllocation);
+  h->n = n;
+  h->from = from;
+  __atomic_add_fetch(&held, n, __ATOMIC_SEQ_CST);
+  *p = h + 1;
+  return cudaSuccess;
+}
+static cudaError_t take(void *p) {
+  struct head *h = p ? (struct head *)p - 1 : 0;
+  if (!h) return cudaSuccess;
+  if (h->from) h->from->idle += h->n;
+  else __atomic_sub_fetch(&held, h->n, __ATOMIC_SEQ_CST);
+  free(h);
+  return cudaSuccess;
+}
+static void trim(struct pool *p, unsigned long long keep) {
+  if (p->idle <= keep) return;
+  __atomic_sub_fetch(&held, p->idle, __ATOMIC_SEQ_CST);
+  p->idle = 0;
 }
 
 /* ---- registration and launches ---- */
@@ -100,13 +124,33 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned f) {
   return cudaSuccess;
 }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { free(s); return cudaSuccess; }
-static void wait_a_while(void) { usleep(300); }
+static void wait_a_while(void) {
+  usleep(300);
+  for (int i = 0; i < n_pools; ++i) trim(pools[i], pools[i]->keep);
+}
 cudaError_t cudaStreamSynchronize(cudaStream_t s) { (void)s; wait_a_while(); return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize(void) { wait_a_while(); return cudaSuccess; }
-cudaError_t cudaMalloc(void **p, size_t n) { return give(p, n); }
-cudaError_t cudaFree(void *p) { free(p); return cudaSuccess; }
-cudaError_t cudaMallocHost(void **p, size_t n) { return give(p, n); }
+cudaError_t cudaMalloc(void **p, size_t n) { return give(p, n, 0); }
+cudaError_t cudaFree(void *p) { return take(p); }
+cudaError_t cudaMallocHost(void **p, size_t n) { return (*p = calloc(1, n)) ? cudaSuccess : ret(cudaErrorMemoryAllocation); }
 cudaError_t cudaFreeHost(void *p) { free(p); return cudaSuccess; }
+cudaError_t cudaMemPoolCreate(cudaMemPool_t *p, const struct cudaMemPoolProps *q) {
+  (void)q;
+  if (n_pools == 16) abort();
+  *p = (cudaMemPool_t)(pools[n_pools++] = calloc(1, sizeof(struct pool)));
+  return cudaSuccess;
+}
+cudaError_t cudaMemPoolDestroy(cudaMemPool_t p) { (void)p; return cudaSuccess; }
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t p, enum cudaMemPoolAttr a, void *v) {
+  if (a == cudaMemPoolAttrReleaseThreshold) ((struct pool *)p)->keep = *(unsigned long long *)v;
+  return cudaSuccess;
+}
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t p, size_t keep) { trim((struct pool *)p, keep); return cudaSuccess; }
+cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t from, cudaStream_t s) {
+  (void)s;
+  return give(p, n, (struct pool *)from);
+}
+cudaError_t cudaFreeAsync(void *p, cudaStream_t s) { (void)s; return take(p); }
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, enum cudaMemcpyKind k) { (void)k; memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, enum cudaMemcpyKind k, cudaStream_t t) {
   (void)k; (void)t;

@@ -79,3 +79,17 @@ rt.cudaGetDevice(ctypes.byref(dev))
 assert dev.value == 1
 print("ok")
 """)
+
+
+def test_stateless_calls_keep_at_most_the_pool_bound(runtime):
+    runtime("""
+rt.fake_device_bytes.restype = ctypes.c_size_t
+keep = 16 << 20
+for n in (64, 60000):  # a gradient of 60000 records takes 53 MB of scratch
+    h4d.h4d_proposal_grad(np.zeros(h4d.H4D_PROP_NW), np.zeros((n, 2, 96), np.float32), np.zeros((n, 2), np.float32))
+    assert rt.fake_device_bytes() <= keep, (n, rt.fake_device_bytes())
+h4d.h4d_proposal_grad(np.zeros(h4d.H4D_PROP_NW), np.zeros((64, 2, 96), np.float32), np.zeros((64, 2), np.float32))
+context(2)[0].close()  # what the pool keeps goes back with a context
+assert rt.fake_device_bytes() == 0
+print("ok")
+""")
