@@ -1,6 +1,7 @@
 // h4d_api.cu -- host side of the libh4d C ABI (declared in include/h4d.h): parameter
 // checking, device buffers, launch plan, state transfer and checkpoints.  All simulation
 // steps run in the kernels of h4d_engine.cu.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -832,7 +833,8 @@ static int upload_replica(h4d_ctx* c, int r, int n_pairs, const double* x, const
 }
 
 namespace h4d {
-// One pool per device, made on first use.  cudaMalloc and cudaFree of a call's buffers took 40 and
+// One pool per CUDA context, made on first use: a pool ends with its context (cudaDeviceReset), and
+// its handle is not used again, so pools are found by the context's id.  cudaMalloc and cudaFree of a call's buffers took 40 and
 // 32 us, a tenth of these calls and more; the pool hands memory out in stream order, so calls
 // from several threads are safe.  It keeps what is freed to it, up to kScratchKeep, and gives more
 // back only at the next wait, which a call does not make after its last free: a call that needs
@@ -841,16 +843,27 @@ namespace h4d {
 // h4d_proposal_grad (4096 records; fifteen allocations before) 490 -> 106 us, the device query of
 // check_device included.
 static std::mutex g_pool_mu;
-static std::map<int, cudaMemPool_t> g_pools;
+static std::map<unsigned long long, cudaMemPool_t> g_pools;
+
+// id of the current context (made if there is none yet), unique for the life of the process
+static bool context_id(unsigned long long* id) {
+  using Fn = CUresult (*)(CUcontext, unsigned long long*);
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+  return cudaFree(nullptr) == cudaSuccess &&
+         cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &found) == cudaSuccess &&
+         found == cudaDriverEntryPointSuccess && reinterpret_cast<Fn>(fn)(nullptr, id) == CUDA_SUCCESS;
+}
 
 int scratch_alloc(void** p, size_t bytes) {
   if (bytes > kScratchKeep) return cudaMalloc(p, bytes) == cudaSuccess ? H4D_OK : H4D_ECUDA;
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return H4D_ECUDA;
+  unsigned long long id = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || !context_id(&id)) return H4D_ECUDA;
   cudaMemPool_t pool = nullptr;
   {
     std::lock_guard<std::mutex> lock(g_pool_mu);
-    auto it = g_pools.find(dev);
+    auto it = g_pools.find(id);
     if (it == g_pools.end()) {
       cudaMemPoolProps props;
       std::memset(&props, 0, sizeof(props));
@@ -863,7 +876,7 @@ int scratch_alloc(void** p, size_t bytes) {
         cudaMemPoolDestroy(pool);
         return H4D_ECUDA;
       }
-      it = g_pools.emplace(dev, pool).first;
+      it = g_pools.emplace(id, pool).first;
     }
     pool = it->second;
   }
@@ -875,12 +888,12 @@ void scratch_free(void* p, size_t bytes) {
   else cudaFreeAsync(p, 0);
 }
 
-// what the pool of the current device still keeps goes back to the device
+// what the pool of the current context still keeps goes back to the device
 static void scratch_trim() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return;
+  unsigned long long id = 0;
+  if (!context_id(&id)) return;
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  const auto it = g_pools.find(dev);
+  const auto it = g_pools.find(id);
   if (it != g_pools.end()) cudaMemPoolTrimTo(it->second, 0);
 }
 }  // namespace h4d

@@ -2,7 +2,11 @@
  * libh4d: two "devices" whose memory is host memory, work done when it is queued, and waits
  * that take a while (so that threads overlap in them).  Kernels do nothing except
  * export_state, which is carried out.  A launch on a stream of another device than the
- * current one is refused, as CUDA does. */
+ * current one is refused, as CUDA does.  A memory pool keeps what is freed to it until the
+ * next wait and then, if that is more than its release threshold, gives it back;
+ * fake_device_bytes() is what the devices hold.  cudaDeviceReset ends the context: a pool
+ * made before it is refused. */
+#include <cuda.h>
 #include <cuda_runtime_api.h>
 #include <stdint.h>
 #include <stdlib.h>
@@ -21,7 +25,8 @@ static cudaError_t ret(cudaError_t e) {
   return e;
 }
 static size_t held;
-struct pool { size_t idle; unsigned long long keep; };
+struct pool { size_t idle; unsigned long long keep; int dead; };
+static unsigned long long ctx_id = 1;
 struct head { size_t n; struct pool *from; char fill[240]; };
 static struct pool *pools[16];
 static int n_pools;
@@ -101,6 +106,19 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void **a, size_t 
 }
 
 /* ---- devices, streams, memory ---- */
+static CUresult ctx_get_id(CUcontext c, unsigned long long *id) { (void)c; *id = ctx_id; return CUDA_SUCCESS; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char *name, void **f, unsigned v, unsigned long long fl,
+                                             enum cudaDriverEntryPointQueryResult *st) {
+  (void)v; (void)fl;
+  *f = strcmp(name, "cuCtxGetId") == 0 ? (void *)ctx_get_id : 0;
+  if (st) *st = *f ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+  return cudaSuccess;
+}
+cudaError_t cudaDeviceReset(void) {
+  for (int i = 0; i < n_pools; ++i) { trim(pools[i], 0); pools[i]->dead = 1; }
+  ++ctx_id;
+  return cudaSuccess;
+}
 cudaError_t cudaGetDeviceCount(int *n) { *n = 2; return cudaSuccess; }
 cudaError_t cudaGetDevice(int *d) { *d = t_dev; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { t_dev = d; return cudaSuccess; }
@@ -148,6 +166,7 @@ cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t p, enum cudaMemPoolAttr a, voi
 cudaError_t cudaMemPoolTrimTo(cudaMemPool_t p, size_t keep) { trim((struct pool *)p, keep); return cudaSuccess; }
 cudaError_t cudaMallocFromPoolAsync(void **p, size_t n, cudaMemPool_t from, cudaStream_t s) {
   (void)s;
+  if (((struct pool *)from)->dead) return ret(cudaErrorInvalidValue);
   return give(p, n, (struct pool *)from);
 }
 cudaError_t cudaFreeAsync(void *p, cudaStream_t s) { (void)s; return take(p); }

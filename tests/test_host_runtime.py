@@ -93,3 +93,17 @@ context(2)[0].close()  # what the pool keeps goes back with a context
 assert rt.fake_device_bytes() == 0
 print("ok")
 """)
+
+
+def test_stateless_calls_work_after_a_device_reset(runtime):
+    runtime("""
+def grad():
+    h4d.h4d_proposal_grad(np.zeros(h4d.H4D_PROP_NW), np.zeros((64, 2, 96), np.float32), np.zeros((64, 2), np.float32))
+
+grad()
+for _ in range(2):
+    rt.cudaDeviceReset()
+    grad()
+    grad()
+print("ok")
+""")
