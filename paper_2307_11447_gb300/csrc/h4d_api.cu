@@ -305,46 +305,93 @@ static int fit_coul_poly(double a, double rc, float* cp) {
 // E^(m)/m! = (2/sqrt pi) (-1)^m I_m / m!, I_m(v) = int_0^1 t^{2m} e^{-v t^2} dt.  Integration by
 // parts gives (2m + 1) I_m = e^{-v} + 2 v I_{m+1}, a sum of positive terms, started at m = 6
 // from the series I_m = e^{-v} / (2m + 1) sum_k v^k / ((m + 3/2)(m + 5/2)...(m + k + 1/2)).
-// A piece spans at most 0.0124 in v, where the first term left out (m = 6) is below 1e-17 and
-// the FP32 terms (m >= 3) below 6e-9 of E(0) (rounded to 4e-16 of it at a piece's ends, less
-// inside).  Energies of LJ and aqueous boxes are within 3e-16 of 80-bit sums, as with erfc;
-// pieces of half the width changed neither that nor the time.
+// A piece spans kPieceV in v: the first term left out (m = 7) is below 2e-20 there, the FP32 ones
+// (m >= 4) below 2e-12.
+// A piece's constant term is shared by all pairs in it, so its rounding does not average out: with
+// plain FP64 coefficients the energy of a 400-water box was off by 1e-13 of itself (3e-15 with
+// erfc).  The series are therefore summed in double-double and the constant term keeps its low
+// part.  They depend on nothing but v: made once per process (0.8 ms on an x86 core), scaled by
+// alpha in coul_table (20 us for 493 pieces).
+constexpr double kPieceV = 13.0 / 1024.0;
+constexpr int kPieces = 993;
+struct CoulSeries {
+  struct { double e0, lo, e[7]; } at[kPieces];  // E (e0 + lo) and E^(m)/m! (e[1..6]) at the pieces' centres
+
+  struct DD { double h, l; };
+  static DD norm(double a, double b) { const double s = a + b; return {s, b - (s - a)}; }  // |a| >= |b|
+  static DD two_sum(double a, double b) {
+    const double s = a + b, t = s - a;
+    return {s, (a - (s - t)) + (b - t)};
+  }
+  static DD add(DD a, DD b) { const DD s = two_sum(a.h, b.h); return norm(s.h, s.l + (a.l + b.l)); }
+  static DD mul(DD a, DD b) {
+    const double p = a.h * b.h;
+    return norm(p, std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+  }
+  static DD div(DD a, double b) { const double q = a.h / b; return norm(q, (std::fma(-q, b, a.h) + a.l) / b); }
+  static DD exp_small(double x) {  // |x| < 0.02
+    DD s = {1.0, 0.0}, t = s;
+    for (int k = 1; k < 16; ++k) s = add(s, t = div(mul(t, {x, 0.0}), k));
+    return s;
+  }
+  CoulSeries() {
+    const DD kC = {1.1283791670955126, 1.5335459613165881e-17};  // 2/sqrt pi
+    const DD step = exp_small(-kPieceV);
+    DD ev = exp_small(-0.5 * kPieceV);
+    for (int k = 0; k < kPieces; ++k, ev = mul(ev, step)) {
+      const double v = (k + 0.5) * kPieceV;  // exact
+      DD t = {1.0, 0.0}, s = t, I[7];
+      for (int q = 1; t.h > 1e-22 * s.h; ++q) s = add(s, t = div(mul(t, {v, 0.0}), q + 6.5));
+      I[6] = div(mul(ev, s), 13.0);
+      for (int m = 5; m >= 0; --m) I[m] = div(add(ev, mul(I[m + 1], {2.0 * v, 0.0})), 2 * m + 1);
+      const DD e0 = mul(kC, I[0]);
+      at[k].e0 = e0.h;
+      at[k].lo = e0.l;
+      double f = kC.h;
+      for (int m = 1; m < 7; ++m) at[k].e[m] = (f /= -m) * I[m].h;
+    }
+  }
+};
+
 static int coul_pieces(double alpha, double rc) {
   const double v = alpha * alpha * rc * rc;
-  if (!(v >= 0) || v > 12.6) return 0;  // over 1024 pieces: the library erfc
-  return std::max(1, (int)std::ceil(v / 0.0123));
+  if (!(v >= 0) || v > 12.6) return 0;  // beyond the pieces: the library erfc
+  return std::max(1, (int)std::ceil(v / kPieceV));
 }
 
 static std::vector<CoulPiece> coul_table(double alpha, double rc) {
+  static const CoulSeries S;
   const int n = coul_pieces(alpha, rc);
   const double shift = std::erfc(alpha * rc) / rc;
   std::vector<CoulPiece> t(std::max(n, 1));
   std::memset(t.data(), 0, t.size() * sizeof(CoulPiece));
+  const double a2 = alpha * alpha, a2_lo = std::fma(alpha, alpha, -a2);
   for (int k = 0; k < n; ++k) {
     CoulPiece& c = t[k];
-    c.sc = (k + 0.5) * (rc * rc / n);
-    const double a2 = alpha * alpha, v = a2 * c.sc, ev = std::exp(-v);
-    double I[7], term = 1.0, sum = 0.0;
-    for (int q = 1; q < 200 && term > 1e-18 * sum; ++q) {
-      sum += term;
-      term *= v / (6.0 + q + 0.5);
+    double e0 = S.at[k].e0, e0_lo = S.at[k].lo, e[7];
+    std::memcpy(e, S.at[k].e, sizeof(e));
+    if (n == 1) {  // alpha^2 s may be tiny or 0 throughout: around s = 0, where I_m = 1 / (2m + 1)
+      e0 = 1.1283791670955126;
+      e0_lo = 1.5335459613165881e-17;
+      double f = e0;
+      for (int m = 1; m < 7; ++m) e[m] = (f /= -m) / (2 * m + 1);
+    } else {
+      const double v = (k + 0.5) * kPieceV;
+      c.sc = v / a2;
+      e0_lo += e[1] * (std::fma(a2, c.sc, -v) + a2_lo * c.sc);  // the centre as rounded
     }
-    I[6] = ev * sum / 13.0;
-    for (int m = 5; m >= 0; --m) I[m] = (ev + 2.0 * v * I[m + 1]) / (2 * m + 1);
-    // minus erf(alpha r)/r; 2 alpha/sqrt(pi) with its rounding error, which all pieces share
-    const double kC = 1.1283791670955126, kClo = 1.5335459613165881e-17;
-    double f = -alpha * kC, cm[6];
-    const double f_lo = std::fma(-alpha, kC, -f) - alpha * kClo;
-    for (int m = 0; m < 6; ++m) {
-      cm[m] = m == 0 ? std::fma(f, I[0], f_lo * I[0] - shift) : f * I[m];
-      f *= -a2 / (m + 1);
-    }
-    c.c0 = cm[0];
+    const double p = alpha * e0, p_lo = std::fma(alpha, e0, -p) + alpha * e0_lo;
+    const CoulSeries::DD c0 = CoulSeries::two_sum(-p, -shift);
+    double f = -alpha, cm[7];
+    for (int m = 1; m < 7; ++m) cm[m] = (f *= a2) * e[m];
+    c.c0 = c0.h;
+    c.lo = (float)(c0.l - p_lo);
     c.c1 = cm[1];
     c.c2 = cm[2];
-    c.c3 = (float)cm[3];
+    c.c3 = cm[3];
     c.c4 = (float)cm[4];
     c.c5 = (float)cm[5];
+    c.c6 = (float)cm[6];
   }
   return t;
 }
@@ -406,13 +453,8 @@ static void fill_pot(const h4d_params& p, Pot& P, Proto& pr) {
   P.coul_poly = (p.system == H4D_SYS_LJ) ? fit_coul_poly(p.alpha, p.rc_coul, P.cpoly) : 0;
   P.lj12 = 12.0f * P.eps4[0];
   P.lj6 = 6.0f * P.eps4[0];
-  for (int k = 0; k < 16; ++k) {
-    const double s6 = P.dsig2[k] * P.dsig2[k] * P.dsig2[k];
-    P.dA6[k] = P.deps4[k] * s6;
-    P.dA12[k] = P.deps4[k] * s6 * s6;
-  }
   P.etab_n = coul_pieces(p.alpha, p.rc_coul);
-  P.etab_invw = P.etab_n > 0 ? (float)(P.etab_n / P.drc2_c) : 0.0f;
+  P.etab_invw = (float)(p.alpha * p.alpha / kPieceV);
   std::memset(&pr, 0, sizeof(pr));
   pr.n_f = p.n_f;
   pr.schedule = p.schedule;

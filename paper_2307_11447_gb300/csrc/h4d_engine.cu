@@ -1606,18 +1606,25 @@ __device__ void negate_velocities(const Ctx& c, int n) {
 // FP64 end-point energies
 // ------------------------------------------------------------------------------------
 // The FP64 pipe of sm_103a takes 64 cycles per warp instruction (2 lanes per clock and SM),
-// so these sums are bound by their number of FP64 instructions alone.  The design keeps that
+// and so do conversions from and to FP64 (in integer arithmetic they take a fifth off an aqueous
+// energy), so these sums are bound by their number of FP64 instructions alone.  The design keeps that
 // number low: a lane scans its row with integer arithmetic for the next pair to evaluate
 // (exact squared distance, cut-off test on it), so every FP64 instruction works on pairs
 // inside the cut-off; a pair belongs to the row of i < j when i + j is odd and of i > j
 // otherwise, which gives every row about half of its pairs (with j > i alone, the first
 // atoms own all of their pairs and the last ones none, and a warp waits for the fullest
-// row); 1/r comes from the FP32 rsqrt and one third-order step; erf(alpha r)/r from a table
-// of short polynomials whose small terms run in FP32; the terms of four pairs are added
-// by the multiply-adds that form them before one compensated addition.  Measured on 304
-// chains of 4000 ions at density 0.3: 2 ms per energy, against 41 ms for rows of j > i with
-// FP64 erfc, square root and divisions per pair; 152 aqueous chains of 9110 atoms: 13 ms
-// against 160 ms.  (ncu on the older form: FP64 pipe 78% busy, half of its lanes idle.)
+// row); 1/r and 1/r^2 come from the FP32 rsqrt and one third-order step; erf(alpha r)/r from a
+// table of short polynomials; what is far below the last bit of a term runs in FP32.
+// No approximation may cost precision: r^2 is the exact integer rounded once, and 1/r -
+// erf(alpha r)/r, which cancel at the cut-off, are added leading part to leading part (the
+// 24-bit rsqrt is exact there) and their corrections apart, so a pair's terms are as good as
+// erfc and divisions make them and every term is added with compensation.
+// Measured against extended precision, rms: six lattices of 1500 waters 0.34 x 2^-53 sum |u| with
+// FP64 erfc, square root and divisions per pair, 0.13 here (3.1 with r^2 from a rounded d2 and table
+// constants of one FP64 word); ten boxes of 1000 ions 1.9e-16, 1.7e-16 and 7.4e-16 of U.
+// Time per energy: 304 chains of 4000 ions at density 0.3 2.3 ms, against 19 ms for rows of j > i
+// with FP64 erfc, square root and divisions per pair; 152 aqueous chains of 9110 atoms 14.6 ms
+// against 159 ms.  (ncu on the older form: FP64 pipe 78% busy, half of its lanes idle.)
 
 // float -> double of a positive normal value (exponent re-bias; exact)
 __device__ __forceinline__ double f2d_pos(float f) {
@@ -1629,6 +1636,12 @@ __device__ __forceinline__ double f2d(float f) {
   const unsigned b = __float_as_uint(f);
   return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
+// double -> float, cut to 24 bits (conversion instructions run on the FP64 pipe); a value below
+// the normal range becomes one below 2^-125
+__device__ __forceinline__ float d2f(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), m = max(hi & 0x7FFFFFFFu, 0x38000000u) - 0x38000000u;
+  return __uint_as_float((hi & 0x80000000u) | (m << 3) | ((unsigned)__double2loint(d) >> 29));
+}
 
 // U over atoms [0, n_tot) leaving out ex0/ex1/ex2 (-1 = none); each unordered pair once
 __device__ H4D_PHASE double energy64_impl(const Ctx& cref, int ex0, int ex1, int ex2);
@@ -1639,29 +1652,51 @@ __device__ double energy64(const Ctx& c, int ex0, int ex1, int ex2 = -1) {
   return u;
 }
 
+// r^2 of an exact squared distance d2 in fixed-point units: d2 (box edge / 2^32)^2, rounded once.
+// (Rounding d2 itself to FP64 would bias the energy: sums of three squares are not evenly
+// spread over their last bits.)
+struct R2Scale {
+  double s;       // the unit squared
+  float sf, slo;  // the same in FP32; 2^32 times its rounding error
+};
+__device__ __forceinline__ R2Scale r2_scale(double L) {
+  const double u = L * 0x1.0p-32, s = u * u;
+  return R2Scale{s, (float)s, (float)(fma(u, u, -s) * 4294967296.0)};
+}
+__device__ __forceinline__ double r2_of(u64 d2, const R2Scale& S) {
+  if (d2 == 0) return 0.0;
+  // the leading 53 bits as FP64, in integer arithmetic, and the remaining ones as FP32
+  const int lz = __clzll((long long)d2);
+  const u64 m = d2 << lz;
+  const double top = __hiloint2double(((1085 - lz) << 20) + (int)(m >> 43), (int)(unsigned)(m >> 11));
+  const float rest = (float)(unsigned)(m & 2047u) * __uint_as_float((unsigned)(127 - lz) << 23);
+  return fma(top, S.s, f2d(fmaf(rest, S.sf, (float)(unsigned)(d2 >> 32) * S.slo)));
+}
+
 // part + the pair energy at r2 (LJ when lj, Coulomb when co), kqg = charge prefactor times
 // the screening
 __device__ __forceinline__ double pair_add64(const Pot& P, const CoulPiece* __restrict__ tab, int k, double r2, double kqg,
                                              bool lj, bool co, double part) {
-  const float sf = (float)r2;
+  const float sf = d2f(r2);
   const float y0 = rsqrt_approx(sf);
-  // r2 = 0 (two atoms on one grid point): 1/r is infinite, as r2 / r2 arithmetic has it
-  const double yd = sf > 1.2e-38f ? f2d_pos(y0) : __hiloint2double(0x7FF00000, 0);
+  // r2 = 0 (two atoms on one grid point): 1/r is infinite
+  const double yd = sf > 1.2e-38f ? f2d_pos(y0) : __hiloint2double(0x7FF00000, 0), yd2 = yd * yd;  // (exact: 48 bits)
   // e = 1 - r2 y0^2 is below 4e-7: 1/r = y0 (1 + e/2 + 3/8 e^2), the next term below 2e-20
-  const double e = fma(-r2, yd * yd, 1.0);
-  const float ef = (float)e;
-  const double y = fma(f2d_pos(0.5f * y0), e + f2d_pos(0.75f * ef * ef), yd);
+  const double e = fma(-r2, yd2, 1.0);
+  const float ef = d2f(e);
   if (lj && __double2hiint(P.deps4[k]) != 0) {  // (tests on the high word: no FP64 compare)
-    const double y2 = y * y, y6 = y2 * y2 * y2;
-    part += fma(fma(P.dA12[k], y6, -P.dA6[k]), y6, -P.dljshift[k]);
+    const double y2 = fma(yd2, e, f2d_pos(y0 * y0 * ef * ef)) + yd2;  // 1/r^2 = y0^2 (1 + e + e^2)
+    const double s2 = P.dsig2[k] * y2, s6 = s2 * s2 * s2;
+    part += fma(P.deps4[k], fma(s6, s6, -s6), -P.dljshift[k]);
   }
   if (co && (__double2hiint(kqg) << 1) != 0) {
     const int m = min((int)(sf * P.etab_invw), P.etab_n - 1);
     const CoulPiece c = tab[m];
     const double h = r2 - c.sc;
-    const float hf = (float)h;
-    const float q = hf * fmaf(hf, fmaf(hf, c.c5, c.c4), c.c3);
-    part = fma(kqg, fma(h, fma(h, c.c2 + f2d(q), c.c1), c.c0) + y, part);
+    const float hf = d2f(h);
+    const float q = hf * fmaf(hf, fmaf(hf, c.c6, c.c5), c.c4);
+    const double corr = fma(f2d_pos(0.5f * y0), e, f2d(fmaf(0.375f * y0 * ef, ef, c.lo)));
+    part = fma(kqg, (c.c0 + yd) + fma(h, fma(h, fma(h, c.c3 + f2d(q), c.c2), c.c1), corr), part);
   }
   return part;
 }
@@ -1673,10 +1708,10 @@ __device__ H4D_PHASE double energy64_impl(const Ctx& cref, int ex0, int ex1, int
   const Pot& P = e.pot;
   const GView& v = c.v;
   const int n = v.s->n_tot;
-  const double scale = R.L * 0x1.0p-32, scale2 = scale * scale;
+  const R2Scale S = r2_scale(R.L);
   const double gscr = exp(-P.dkappa_sr * (double)v.s->w_cur);
   // cut-offs on exact squared distances in fixed-point units
-  const u64 T_lj = (u64)ceil(P.drc2_lj / scale2), T_c = (u64)ceil(P.drc2_c / scale2);
+  const u64 T_lj = (u64)ceil(P.drc2_lj / S.s), T_c = (u64)ceil(P.drc2_c / S.s);
   const u64 T_max = T_lj > T_c ? T_lj : T_c;
   // per-atom sums over the row, then a sum over atoms in a fixed order; rows are taken by
   // position k (atom ord[k])
@@ -1691,8 +1726,8 @@ __device__ H4D_PHASE double energy64_impl(const Ctx& cref, int ex0, int ex1, int
     const int ti = type_of(i, R.nw3);
     const float wi = wbits(pi);
     const int cnt = own ? e.ncnt[R.atom_off + k] : 0;
-    double acc = 0.0, comp = 0.0, part = 0.0;
-    int s = 0, np = 0;
+    double acc = 0.0, comp = 0.0;
+    int s = 0;
     uint2 q = make_uint2(0u, 0u);
     for (;;) {
       bool have = false;
@@ -1714,31 +1749,27 @@ __device__ H4D_PHASE double energy64_impl(const Ctx& cref, int ex0, int ex1, int
       if (!__any_sync(0xffffffffu, have)) break;
       if (have) {
         const int tk = ti * 4 + type_of(j, R.nw3);
-        double r2 = __ull2double_rn(d2) * scale2;
-        double kqg = P.dkq[tk];
+        double r2 = r2_of(d2, S), g = 1.0, kqg = P.dkq[tk];
         bool lj = d2 < T_lj, co = d2 < T_c;
         if (wi != wj) {  // altitudes differ: one of the two flies
           const double dw = (double)wi - (double)wj;
           r2 = fma(dw, dw, r2);
           lj = r2 < P.drc2_lj;
           co = r2 < P.drc2_c;
-          if ((wi != 0.f) != (wj != 0.f)) kqg *= gscr;
+          if ((wi != 0.f) != (wj != 0.f)) {
+            g = gscr;
+            kqg *= g;
+          }
         }
-        if (P.etab_n > 0) {
-          part = pair_add64(P, e.etab, tk, r2, kqg, lj, co, part);
-        } else {
-          part += pair_u64(P, ti, tk - 4 * ti, r2, P.dkq[tk] != 0.0 ? kqg / P.dkq[tk] : 1.0);
-        }
-        if (++np == 4) {
-          const double y = part - comp, t = acc + y;
-          comp = (t - acc) - y;
-          acc = t;
-          part = 0.0;
-          np = 0;
-        }
+        // Kahan's sum; the pair's terms are added to minus the compensation
+        const double y = P.etab_n > 0 ? pair_add64(P, e.etab, tk, r2, kqg, lj, co, -comp)
+                                      : pair_u64(P, ti, tk - 4 * ti, r2, g) - comp;
+        const double t = acc + y;
+        comp = (t - acc) - y;
+        acc = t;
       }
     }
-    if (act) e.red[R.atom_off + i] = acc + (part - comp);
+    if (act) e.red[R.atom_off + i] = acc;
   }
   return fixed_order_sum(c, e.red + R.atom_off, n);
 }
@@ -3122,14 +3153,14 @@ __global__ void __launch_bounds__(512) point_kernel(const __grid_constant__ Poin
   __syncthreads();
   const Pot& P = a.pot;
   const float scale = (float)(a.L / 4294967296.0);
-  const double dscale = a.L * 0x1.0p-32, scale2 = dscale * dscale;
+  const R2Scale S = r2_scale(a.L);
   const float gscr = expf(-P.kappa_sr * a.wbar);
   const double gscr64 = exp(-P.dkappa_sr * (double)a.wbar);
-  const u64 T_lj = (u64)ceil(P.drc2_lj / scale2), T_c = (u64)ceil(P.drc2_c / scale2);
+  const u64 T_lj = (u64)ceil(P.drc2_lj / S.s), T_c = (u64)ceil(P.drc2_c / S.s);
   const u64 T_max = T_lj > T_c ? T_lj : T_c;
   const unsigned lt = (1u << lane) - 1u;
   const int w0 = (blockIdx.x * nwarps + warp) * a.homes;
-  double part = 0.0;
+  double part = 0.0, comp = 0.0;
   for (int i = w0; i < min(w0 + a.homes, a.n); ++i) {
     const uint4 pi = pos[i];
     const int ti = type_t<SYS>(i, a.nw3);
@@ -3171,7 +3202,7 @@ __global__ void __launch_bounds__(512) point_kernel(const __grid_constant__ Poin
         if (q == 0) {
           const int tk = ti * 4 + tj;
           const u64 d2 = fixed_d2(pi, pj);
-          double r264 = __ull2double_rn(d2) * scale2;
+          double r264 = r2_of(d2, S);
           double kqg = P.dkq[tk];
           bool lj = d2 < T_lj, co = d2 < T_c;
           if (wi != wj) {
@@ -3181,8 +3212,11 @@ __global__ void __launch_bounds__(512) point_kernel(const __grid_constant__ Poin
             co = r264 < P.drc2_c;
             if (screened) kqg *= gscr64;
           }
-          if (P.etab_n > 0) part = pair_add64(P, a.etab, tk, r264, kqg, lj, co, part);
-          else part += pair_u64(P, ti, tj, r264, screened ? gscr64 : 1.0);
+          const double y = P.etab_n > 0 ? pair_add64(P, a.etab, tk, r264, kqg, lj, co, -comp)
+                                        : pair_u64(P, ti, tj, r264, screened ? gscr64 : 1.0) - comp;
+          const double t = part + y;  // Kahan's sum over the lane's pairs
+          comp = (t - part) - y;
+          part = t;
         }
       }
       __syncwarp();

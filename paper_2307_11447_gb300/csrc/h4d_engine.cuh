@@ -40,19 +40,18 @@ struct Pot {
   int coul_poly;
   float cpoly[8];
   float lj12, lj6;      // 12 eps4 and 6 eps4 of the LJ electrolyte (one sigma, one epsilon)
-  // FP64 energies: LJ term dA12 r^-12 - dA6 r^-6, Coulomb term from a table of erf(alpha r)/r
-  // over s = r^2 with etab_n pieces of width 1 / etab_invw (0: the library erfc)
-  double dA12[16], dA6[16];
+  // FP64 energies: Coulomb term from a table of erf(alpha r)/r over s = r^2 with etab_n pieces of
+  // width 1 / etab_invw (0: the library erfc)
   int etab_n;
   float etab_invw;
 };
 
 // One piece of the FP64 Coulomb table: -(erf(alpha r)/r) - shift as a polynomial in
-// h = s - sc, s = r^2: c0 + c1 h + c2 h^2 in FP64, the h^3..h^5 terms (below 6e-9 of c0) in
-// FP32
+// h = s - sc, s = r^2: c0 + lo + c1 h + c2 h^2 + c3 h^3 in FP64 (lo: what rounding c0 left out), the
+// h^4..h^6 terms (below 2e-12 of c0) in FP32
 struct __align__(16) CoulPiece {
-  double c0, c1, c2, sc;
-  float c3, c4, c5, pad;
+  double c0, c1, c2, c3, sc;
+  float lo, c4, c5, c6;
 };
 
 struct Proto {
