@@ -1938,7 +1938,7 @@ extern "C" int h4d_eval_forces(const h4d_params* params, double L, int32_t n_wat
   double u = 0.0, comp = 0.0;
   for (int k = 0; k < n_part; ++k) {
     const double y = res[1 + k] - comp, t = u + y;
-    comp = (t - u) - y;
+    comp = std::isfinite(t) ? (t - u) - y : 0.0;
     u = t;
   }
   if (U) *U = u;

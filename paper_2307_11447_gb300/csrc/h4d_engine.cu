@@ -1696,7 +1696,9 @@ __device__ __forceinline__ double pair_add64(const Pot& P, const CoulPiece* __re
     const float hf = d2f(h);
     const float q = hf * fmaf(hf, fmaf(hf, c.c6, c.c5), c.c4);
     const double corr = fma(f2d_pos(0.5f * y0), e, f2d(fmaf(0.375f * y0 * ef, ef, c.lo)));
-    part = fma(kqg, (c.c0 + yd) + fma(h, fma(h, fma(h, c.c3 + f2d(q), c.c2), c.c1), corr), part);
+    double w = (c.c0 + yd) + fma(h, fma(h, fma(h, c.c3 + f2d(q), c.c2), c.c1), corr);
+    if (!(sf > 1.2e-38f)) w = yd;  // (its correction is NaN there)
+    part = fma(kqg, w, part);
   }
   return part;
 }
