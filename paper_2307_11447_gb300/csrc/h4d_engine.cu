@@ -1108,15 +1108,21 @@ __device__ __forceinline__ void aq_row(const Pot& P, const uint4* __restrict__ p
 // mode bits: 1 = apply the second half kick, 2 = accumulate kinetic partials,
 //            4 = flyer rows compute protocol work with previous altitude w_prev
 // ------------------------------------------------------------------------------------
-template <int SYS, bool NEMD>
+template <int SYS, bool NEMD, bool PARTS>
 __device__ H4D_PHASE void force_pass_impl(const Ctx& cref, int mode, float w_prev, double* kin_out);
 // mode bits: 1 = apply the second half kick, 2 = return the kinetic energy after it,
 //            4 = flyer rows accumulate the protocol work between w_prev and the current w.
 // NEMD = false assumes every altitude is zero (equilibrium MD).
-template <int SYS, bool NEMD = true>
+// PARTS = false takes no account of lanes < tpa (the sums are the same bits).  The loop over parts
+// is compiled apart from the plain pass: in one function, with the number of parts known at run
+// time only, it cost the plain pass spills.  Force pass inside the engine, 304 chains of 250 ions on
+// 1 / 4 / 16 lanes 11.1 / 10.2 / 20.9 -> 10.1 / 8.7 / 16.7 us, of 4000 ions on 1 / 8 lanes 186 / 363 ->
+// 180 / 319 us.
+template <int SYS, bool NEMD = true, bool PARTS = SYS == H4D_SYS_LJ>
 __device__ void force_pass(const Ctx& c, int mode, float w_prev, double* kin_out) {
   const u64 t0 = (c.tid == 0) ? gtimer() : 0;
-  force_pass_impl<SYS, NEMD>(c, mode, w_prev, kin_out);
+  if (PARTS && c.llan != c.ltpa) force_pass_impl<SYS, NEMD, true>(c, mode, w_prev, kin_out);
+  else force_pass_impl<SYS, NEMD, false>(c, mode, w_prev, kin_out);
   if (c.tid == 0) c.R->t_force_ns += (double)(gtimer() - t0);
 }
 
@@ -1160,7 +1166,8 @@ __device__ __forceinline__ void protocol_work(const Ctx& c, int i, int k, float 
   if ((c.tid & 31) == 0) v.s->dW[i == fly0 ? 0 : (i == fly1 ? 1 : 2)] = (double)dw;
 }
 
-template <int SYS, bool NEMD>
+// PARTS: a lane takes several parts of its row (lanes < tpa)
+template <int SYS, bool NEMD, bool PARTS>
 __device__ H4D_PHASE void force_pass_impl(const Ctx& cref, int mode, float w_prev, double* kin_out) {
   const Ctx c = cref;
   const Eng& e = *c.e;
@@ -1168,7 +1175,7 @@ __device__ H4D_PHASE void force_pass_impl(const Ctx& cref, int mode, float w_pre
   const Pot& P = e.pot;
   const GView& v = c.v;
   const int n = v.s->n_tot;
-  const int tpa = c.tpa, ltpa = c.ltpa, llan = c.llan;
+  const int tpa = c.tpa, ltpa = c.ltpa, llan = PARTS ? c.llan : c.ltpa;
   const int nsub = c.T >> llan;
   const int sub = c.tid >> llan, lin = c.tid & ((1 << llan) - 1);
   const int fly0 = NEMD ? v.s->fly0 : -1, fly1 = NEMD ? v.s->fly1 : -1, fly2 = NEMD ? v.s->fly2 : -1;
@@ -1204,8 +1211,18 @@ __device__ H4D_PHASE void force_pass_impl(const Ctx& cref, int mode, float w_pre
       const int nP = (cnt + 3) >> 2;  // packets of the row, dealt to tpa parts: part l owns l, l+tpa, ...
       int npk = (nP > lin) ? (nP - lin + tpa - 1) >> ltpa : 0;
       uint2 q = (npk > 0) ? pk[0] : make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
-      if (SYS == H4D_SYS_LJ) {
-        // A lane takes 1, 2 or 4 parts, in the order in which a butterfly over tpa lanes adds
+      const auto row = [&]() {
+        if (P.coul_poly && P.rc2_lj <= P.rc2_c)
+          lj_row<NEMD, 1>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
+        else if (P.coul_poly)
+          lj_row<NEMD, 2>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
+        else
+          lj_row<NEMD, 0>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
+      };
+      if (SYS == H4D_SYS_LJ && !PARTS) {
+        row();
+      } else if (SYS == H4D_SYS_LJ) {
+        // A lane takes 2 or 4 parts, in the order in which a butterfly over tpa lanes adds
         // them: the sum is the same bits with fewer lanes
         const int lnv = ltpa - llan;
         float s0x = 0.f, s0y = 0.f, s0z = 0.f, s1x = 0.f, s1y = 0.f, s1z = 0.f;
@@ -1218,12 +1235,7 @@ __device__ H4D_PHASE void force_pass_impl(const Ctx& cref, int mode, float w_pre
           uint2 qn = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
           if (npn > 0) qn = ld_packet(pkn);
           fx = fy = fz = 0.f;
-          if (P.coul_poly && P.rc2_lj <= P.rc2_c)
-            lj_row<NEMD, 1>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
-          else if (P.coul_poly)
-            lj_row<NEMD, 2>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
-          else
-            lj_row<NEMD, 0>(P, v.pos, pk, pstride, npk, q, i, pi, scale, wi, wnz_i, gscr, fx, fy, fz);
+          row();
           if (t & 1) {
             fx += s0x; fy += s0y; fz += s0z;
             if (t & 2) { fx += s1x; fy += s1y; fz += s1z; }
@@ -3297,7 +3309,7 @@ __global__ void __launch_bounds__(H4D_MAXTHREADS, H4D_MINBLOCKS) forces_kernel(c
   if (!setup_ctx(e, smem, c)) return;
   build_list(c);
   for (int it = 0; it < n_iter; ++it) {
-    force_pass<SYS, false>(c, 0, 0.f, nullptr);
+    force_pass<SYS, false, false>(c, 0, 0.f, nullptr);
     c.sync();
   }
 }
