@@ -2013,9 +2013,14 @@ extern "C" int h4d_eval_forces_static(const h4d_params* params, double L, int32_
   const size_t o_red = carve_bytes(off, na * sizeof(double));
   std::memset(&c.eng, 0, sizeof(Eng));
   fill_pot(c.prm, c.eng.pot, c.eng.proto);
-  const std::vector<CoulPiece> etab = coul_table(c.prm.alpha, c.prm.rc_coul);
-  const size_t o_tab = carve_bytes(off, etab.size() * sizeof(CoulPiece));
   if (off > kStaticScratchBytes) return H4D_ECAPACITY;  // too many atoms for 16 MiB
+  // The energies' Coulomb table goes where there is room for it; the last few sizes (6220 and 6222
+  // LJ atoms with altitudes, at default capacities) take the library erfc instead
+  const std::vector<CoulPiece> etab = coul_table(c.prm.alpha, c.prm.rc_coul);
+  size_t end = off;
+  const size_t o_tab = carve_bytes(end, etab.size() * sizeof(CoulPiece));
+  const bool use_tab = end <= kStaticScratchBytes;
+  if (!use_tab) c.eng.pot.etab_n = 0;
 
   unsigned char* b = static_cast<unsigned char*>(base);
   Eng& e = c.eng;
@@ -2052,7 +2057,8 @@ extern "C" int h4d_eval_forces_static(const h4d_params* params, double L, int32_
   if (cudaMemcpy(b + o_rep, &R, sizeof(Rep), cudaMemcpyHostToDevice) != cudaSuccess) return H4D_ECUDA;
   if (cudaMemcpy(b + o_grp, &G, sizeof(Group), cudaMemcpyHostToDevice) != cudaSuccess) return H4D_ECUDA;
   if (cudaMemcpy(b + o_cg, cta_groups, sizeof(cta_groups), cudaMemcpyHostToDevice) != cudaSuccess) return H4D_ECUDA;
-  if (cudaMemcpy(b + o_tab, etab.data(), etab.size() * sizeof(CoulPiece), cudaMemcpyHostToDevice) != cudaSuccess)
+  if (use_tab &&
+      cudaMemcpy(b + o_tab, etab.data(), etab.size() * sizeof(CoulPiece), cudaMemcpyHostToDevice) != cudaSuccess)
     return H4D_ECUDA;
   if (cudaMemcpy(b + o_x, x, na * 3 * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) return H4D_ECUDA;
   if (w && cudaMemcpy(b + o_w, w, na * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) return H4D_ECUDA;
