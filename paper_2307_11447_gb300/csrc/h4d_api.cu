@@ -1596,6 +1596,8 @@ int h4d_load(h4d_ctx* c, const char* path) {
   ok = ok && std::fread(rec.data(), sizeof(h4d_record), nrec, f) == nrec;
   std::fclose(f);
   if (!ok) return H4D_EINVAL;
+  int rc = pull_reps(c);  // what is kept of each replica, as the device has it
+  if (rc) return rc;
   for (int r = 0; r < c->R; ++r) {
     const Rep& cur = c->rep_h[r];
     const Rep& f = reps[r];
@@ -1647,7 +1649,7 @@ int h4d_load(h4d_ctx* c, const char* path) {
   CK(cudaMemcpyAsync(c->d_vhi, vh.data(), na * sizeof(float4), cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemcpyAsync(c->d_vlo, vl.data(), na * sizeof(float4), cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemcpyAsync(c->d_rec, rec.data(), nrec * sizeof(h4d_record), cudaMemcpyHostToDevice, c->stream));
-  int rc = push_plan(c);
+  rc = push_plan(c);
   if (rc) return rc;
   CK(cudaStreamSynchronize(c->stream));
   return H4D_OK;
