@@ -527,6 +527,12 @@ static int choose_lanes(const h4d_params& p, int tpa) {
   return p.threads_per_atom > 0 || p.system != H4D_SYS_LJ ? tpa : std::min(tpa, 4);
 }
 
+// whether the force pass takes rows of tpa parts on this many lanes
+static bool lanes_fit(const h4d_params& p, int tpa, int lanes) {
+  return lanes >= 1 && lanes <= tpa && (lanes & (lanes - 1)) == 0 &&
+         (lanes == tpa || (p.system == H4D_SYS_LJ && 4 * lanes >= tpa));
+}
+
 static int choose_threads(int n_atoms) {
   if (n_atoms >= 2048) return 512;
   if (n_atoms >= 256) return 256;
@@ -1616,7 +1622,10 @@ int h4d_load(h4d_ctx* c, const char* path) {
     m.n_pairs = f.n_pairs;
     m.n_water = f.n_water;
     m.nw3 = f.nw3;
-    if (f.tpa != m.tpa) m.lanes = f.tpa;
+    if (f.tpa != m.tpa) {
+      m.lanes = lanes_fit(c->prm, f.tpa, f.lanes) ? f.lanes : choose_lanes(c->prm, f.tpa);
+      if (!lanes_fit(c->prm, f.tpa, m.lanes)) m.lanes = f.tpa;
+    }
     m.tpa = f.tpa;
     m.rec_count = f.rec_count;
     m.trial_ctr = f.trial_ctr;
