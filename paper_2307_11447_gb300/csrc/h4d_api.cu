@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <tuple>
@@ -758,9 +759,13 @@ static int export_to_host(h4d_ctx* c, size_t bytes, std::vector<unsigned char>& 
     *p = pin;
     return H4D_OK;
   }
+  try {
+    own.resize(bytes);
+  } catch (const std::bad_alloc&) {
+    return H4D_ECUDA;
+  }
   unsigned char* tmp = nullptr;
   CK(cudaMalloc(&tmp, bytes));
-  own.resize(bytes);
   launch(tmp);
   const bool good = cudaGetLastError() == cudaSuccess &&
                     cudaMemcpyAsync(own.data(), tmp, bytes, cudaMemcpyDeviceToHost, c->stream) == cudaSuccess &&
@@ -924,7 +929,12 @@ int scratch_alloc(void** p, size_t bytes) {
         cudaMemPoolDestroy(pool);
         return H4D_ECUDA;
       }
-      it = g_pools.emplace(id, pool).first;
+      try {
+        it = g_pools.emplace(id, pool).first;
+      } catch (const std::bad_alloc&) {
+        cudaMemPoolDestroy(pool);
+        return H4D_ECUDA;
+      }
     }
     pool = it->second;
   }
@@ -1090,6 +1100,60 @@ const char* h4d_strerror(int code) {
   }
 }
 
+// host tables, device buffers and initial states of a new context
+static int fill_context(h4d_ctx* c, const h4d_params* params, const h4d_system* sys) {
+  c->R = sys->n_replicas;
+  c->max_nbr = params->max_nbr > 0 ? params->max_nbr : derive_max_nbr(*params);
+  c->rep_h.resize(c->R);
+  int off = 0;
+  for (int r = 0; r < c->R; ++r) {
+    Rep& R = c->rep_h[r];
+    std::memset(&R, 0, sizeof(Rep));
+    int nw = sys->n_water ? sys->n_water[r] : 0;
+    int cw = sys->cap_water ? sys->cap_water[r] : nw;
+    if (nw < 0 || cw < nw || sys->n_pairs[r] < 0 || sys->cap_pairs[r] < sys->n_pairs[r] || !(sys->L[r] > 0))
+      return H4D_EINVAL;
+    if (cw > 0 && params->system != H4D_SYS_AQ) return H4D_EINVAL;
+    if (cw != nw && params->exchange != H4D_EXCHANGE_WATER) return H4D_EINVAL;
+    R.n_water = nw;
+    R.nw3 = 3 * nw;
+    R.cap_water = cw;
+    R.n_pairs = sys->n_pairs[r];
+    R.cap_pairs = sys->cap_pairs[r];
+    R.cap_atoms = 3 * cw + unit_of(*params) * R.cap_pairs;
+    if (R.cap_atoms > 65535 || R.cap_atoms < 1) return H4D_ECAPACITY;
+    if (2.0 * (rmax_of(*params) + params->skin) >= sys->L[r]) return H4D_EINVAL;
+    R.atom_off = off;
+    off += R.cap_atoms;
+    R.key = sys->replica_key ? sys->replica_key[r] : (uint64_t)r;
+    set_rep_geometry(*params, R, sys->L[r]);
+    R.tpa = choose_tpa(*params, R.cap_atoms);
+    R.lanes = choose_lanes(*params, R.tpa);
+    R.rec_cap = 1024;
+    R.rec_off = r * R.rec_cap;
+  }
+  c->total_atoms = off;
+  // rows are packed 4 per lane and tpa-interleaved: capacity is a multiple of 4 * 32
+  c->max_nbr = ((c->max_nbr + 127) / 128) * 128;
+  c->max_out = std::max(c->max_nbr, derive_max_rows(*params, rmax_of(*params) + outer_skin(*params)));
+  int rc = make_plan(c);
+  if (rc) return rc;
+  rc = alloc_all(c);
+  if (rc) return rc;
+  fill_eng(c);
+  size_t xo = 0;
+  for (int r = 0; r < c->R; ++r) {
+    Rep& R = c->rep_h[r];
+    rc = upload_replica(c, r, R.n_pairs, sys->host_x + xo, sys->host_v ? sys->host_v + xo : nullptr);
+    if (rc) return rc;
+    xo += 3 * (size_t)(R.nw3 + unit_of(*params) * R.n_pairs);
+  }
+  rc = push_plan(c);
+  if (rc) return rc;
+  if (cudaStreamSynchronize(c->stream) != cudaSuccess) return H4D_ECUDA;
+  return H4D_OK;
+}
+
 int h4d_create(const h4d_params* params, const h4d_system* sys, uint64_t seed, void* cuda_stream, h4d_ctx** out) {
   if (!out) return H4D_EINVAL;
   *out = nullptr;
@@ -1114,57 +1178,15 @@ int h4d_create(const h4d_params* params, const h4d_system* sys, uint64_t seed, v
       c->sm_count = prop.multiProcessorCount;
     c->device = dev;
   }
-  c->R = sys->n_replicas;
-  c->max_nbr = params->max_nbr > 0 ? params->max_nbr : derive_max_nbr(*params);
-  c->rep_h.resize(c->R);
-  int off = 0;
-  for (int r = 0; r < c->R; ++r) {
-    Rep& R = c->rep_h[r];
-    std::memset(&R, 0, sizeof(Rep));
-    int nw = sys->n_water ? sys->n_water[r] : 0;
-    int cw = sys->cap_water ? sys->cap_water[r] : nw;
-    if (nw < 0 || cw < nw || sys->n_pairs[r] < 0 || sys->cap_pairs[r] < sys->n_pairs[r] || !(sys->L[r] > 0)) {
-      h4d_destroy(c);
-      return H4D_EINVAL;
-    }
-    if (cw > 0 && params->system != H4D_SYS_AQ) { h4d_destroy(c); return H4D_EINVAL; }
-    if (cw != nw && params->exchange != H4D_EXCHANGE_WATER) { h4d_destroy(c); return H4D_EINVAL; }
-    R.n_water = nw;
-    R.nw3 = 3 * nw;
-    R.cap_water = cw;
-    R.n_pairs = sys->n_pairs[r];
-    R.cap_pairs = sys->cap_pairs[r];
-    R.cap_atoms = 3 * cw + unit_of(*params) * R.cap_pairs;
-    if (R.cap_atoms > 65535 || R.cap_atoms < 1) { h4d_destroy(c); return H4D_ECAPACITY; }
-    if (2.0 * (rmax_of(*params) + params->skin) >= sys->L[r]) { h4d_destroy(c); return H4D_EINVAL; }
-    R.atom_off = off;
-    off += R.cap_atoms;
-    R.key = sys->replica_key ? sys->replica_key[r] : (uint64_t)r;
-    set_rep_geometry(*params, R, sys->L[r]);
-    R.tpa = choose_tpa(*params, R.cap_atoms);
-    R.lanes = choose_lanes(*params, R.tpa);
-    R.rec_cap = 1024;
-    R.rec_off = r * R.rec_cap;
+  try {
+    rc = fill_context(c, params, sys);
+  } catch (const std::bad_alloc&) {
+    rc = H4D_ECUDA;
   }
-  c->total_atoms = off;
-  // rows are packed 4 per lane and tpa-interleaved: capacity is a multiple of 4 * 32
-  c->max_nbr = ((c->max_nbr + 127) / 128) * 128;
-  c->max_out = std::max(c->max_nbr, derive_max_rows(*params, rmax_of(*params) + outer_skin(*params)));
-  rc = make_plan(c);
-  if (rc) { h4d_destroy(c); return rc; }
-  rc = alloc_all(c);
-  if (rc) { h4d_destroy(c); return rc; }
-  fill_eng(c);
-  size_t xo = 0;
-  for (int r = 0; r < c->R; ++r) {
-    Rep& R = c->rep_h[r];
-    rc = upload_replica(c, r, R.n_pairs, sys->host_x + xo, sys->host_v ? sys->host_v + xo : nullptr);
-    if (rc) { h4d_destroy(c); return rc; }
-    xo += 3 * (size_t)(R.nw3 + unit_of(*params) * R.n_pairs);
+  if (rc) {
+    h4d_destroy(c);
+    return rc;
   }
-  rc = push_plan(c);
-  if (rc) { h4d_destroy(c); return rc; }
-  if (cudaStreamSynchronize(c->stream) != cudaSuccess) { h4d_destroy(c); return H4D_ECUDA; }
   *out = c;
   return H4D_OK;
 }
@@ -1674,6 +1696,7 @@ static int eval_forces_lists(const h4d_params* params, double L, int32_t n_water
   int rc;
   h4d_ctx* c = new (std::nothrow) h4d_ctx();
   if (!c) return H4D_ECUDA;
+  const std::unique_ptr<h4d_ctx, void (*)(h4d_ctx*)> owner(c, h4d_destroy);
   c->prm = *params;
   c->seed = 0;
   c->stream = 0;
@@ -1697,9 +1720,9 @@ static int eval_forces_lists(const h4d_params* params, double L, int32_t n_water
   R.rec_cap = 1;
   c->total_atoms = R.cap_atoms;
   rc = make_plan(c);
-  if (rc) { delete c; return rc; }
+  if (rc) return rc;
   rc = alloc_all(c);
-  if (rc) { h4d_destroy(c); return rc; }
+  if (rc) return rc;
   fill_eng(c);
   std::vector<uint4> pos(n);
   double wsum = 0.0;
@@ -1728,7 +1751,6 @@ static int eval_forces_lists(const h4d_params* params, double L, int32_t n_water
     }
     if (U) *U = u;
   }
-  h4d_destroy(c);
   return rc;
 }
 
@@ -1910,7 +1932,15 @@ extern "C" int h4d_eval_forces(const h4d_params* params, double L, int32_t n_wat
   P.wbar = (float)(wcnt ? wsum / wcnt : 0.0);
   int warps, ctas;
   const int n_part = point_plan(n, &warps, &P.homes, &ctas);
-  const std::vector<CoulPiece> tab = coul_table(params->alpha, params->rc_coul);
+  const size_t n_out = 1 + (size_t)n_part + 3 * (size_t)n;
+  std::vector<CoulPiece> tab;
+  std::vector<double> res;
+  try {
+    tab = coul_table(params->alpha, params->rc_coul);
+    res.resize(n_out);
+  } catch (const std::bad_alloc&) {
+    return H4D_ECUDA;
+  }
   // one allocation; inputs and results are each one piece
   const size_t na = (size_t)n;
   size_t off = 0;
@@ -1918,7 +1948,6 @@ extern "C" int h4d_eval_forces(const h4d_params* params, double L, int32_t n_wat
   const size_t o_w = carve_bytes(off, w ? na * sizeof(double) : 0);
   const size_t o_tab = carve_bytes(off, tab.size() * sizeof(CoulPiece));
   const size_t o_pos = carve_bytes(off, na * sizeof(uint4));
-  const size_t n_out = 1 + (size_t)n_part + 3 * na;
   const size_t o_out = carve_bytes(off, n_out * sizeof(double));
   void* slab = nullptr;
   if (scratch_alloc(&slab, off) != H4D_OK) return H4D_ECUDA;
@@ -1929,7 +1958,6 @@ extern "C" int h4d_eval_forces(const h4d_params* params, double L, int32_t n_wat
   P.may_overflow = out;
   P.u_part = out + 1;
   P.F = out + 1 + n_part;
-  std::vector<double> res(n_out);
   auto ok = [](cudaError_t e) { return e == cudaSuccess; };
   bool good = ok(cudaMemcpyAsync(b + o_x, x, na * 3 * sizeof(double), cudaMemcpyHostToDevice, 0));
   if (w) good = good && ok(cudaMemcpyAsync(b + o_w, w, na * sizeof(double), cudaMemcpyHostToDevice, 0));
@@ -1945,7 +1973,13 @@ extern "C" int h4d_eval_forces(const h4d_params* params, double L, int32_t n_wat
   if (!good) cudaStreamSynchronize(0);
   scratch_free(b, off);
   if (!good) return H4D_ECUDA;
-  if (res[0] != 0.0) return eval_forces_lists(params, L, n_water, n, x, w, F, U);
+  if (res[0] != 0.0) {
+    try {
+      return eval_forces_lists(params, L, n_water, n, x, w, F, U);
+    } catch (const std::bad_alloc&) {
+      return H4D_ECUDA;
+    }
+  }
   double u = 0.0, comp = 0.0;
   for (int k = 0; k < n_part; ++k) {
     const double y = res[1 + k] - comp, t = u + y;
@@ -2027,7 +2061,12 @@ extern "C" int h4d_eval_forces_static(const h4d_params* params, double L, int32_
   if (off > kStaticScratchBytes) return H4D_ECAPACITY;  // too many atoms for 16 MiB
   // The energies' Coulomb table goes where there is room for it; the last few sizes (6220 and 6222
   // LJ atoms with altitudes, at default capacities) take the library erfc instead
-  const std::vector<CoulPiece> etab = coul_table(c.prm.alpha, c.prm.rc_coul);
+  std::vector<CoulPiece> etab;
+  try {
+    etab = coul_table(c.prm.alpha, c.prm.rc_coul);
+  } catch (const std::bad_alloc&) {
+    return H4D_ECUDA;
+  }
   size_t end = off;
   const size_t o_tab = carve_bytes(end, etab.size() * sizeof(CoulPiece));
   const bool use_tab = end <= kStaticScratchBytes;

@@ -5,7 +5,8 @@
  * current one is refused, as CUDA does.  A memory pool keeps what is freed to it until the
  * next wait and then, if that is more than its release threshold, gives it back;
  * fake_device_bytes() is what the devices hold.  cudaDeviceReset ends the context: a pool
- * made before it is refused. */
+ * made before it is refused.  fake_fail_new(k) makes this thread's k-th C++ allocation from then on
+ * throw (-1: none), fake_fail_pinned(1) every allocation of pinned memory fail. */
 #include <cuda.h>
 #include <cuda_runtime_api.h>
 #include <stdint.h>
@@ -52,6 +53,16 @@ static void trim(struct pool *p, unsigned long long keep) {
   if (p->idle <= keep) return;
   __atomic_sub_fetch(&held, p->idle, __ATOMIC_SEQ_CST);
   p->idle = 0;
+}
+
+static __thread int new_left = -1;
+static int no_pinned;
+void _ZSt17__throw_bad_allocv(void);
+void fake_fail_new(int k) { new_left = k; }
+void fake_fail_pinned(int on) { no_pinned = on; }
+void *_Znwm(size_t n) {
+  if (new_left >= 0 && new_left-- == 0) _ZSt17__throw_bad_allocv();
+  return malloc(n);
 }
 
 /* ---- registration and launches ---- */
@@ -150,7 +161,15 @@ cudaError_t cudaStreamSynchronize(cudaStream_t s) { (void)s; wait_a_while(); ret
 cudaError_t cudaDeviceSynchronize(void) { wait_a_while(); return cudaSuccess; }
 cudaError_t cudaMalloc(void **p, size_t n) { return give(p, n, 0); }
 cudaError_t cudaFree(void *p) { return take(p); }
-cudaError_t cudaMallocHost(void **p, size_t n) { return (*p = calloc(1, n)) ? cudaSuccess : ret(cudaErrorMemoryAllocation); }
+cudaError_t cudaMallocHost(void **p, size_t n) {
+  return !no_pinned && (*p = calloc(1, n)) ? cudaSuccess : ret(cudaErrorMemoryAllocation);
+}
+cudaError_t cudaGetSymbolAddress(void **p, const void *s) {
+  (void)s;
+  static char array[16 << 20];
+  *p = array;
+  return cudaSuccess;
+}
 cudaError_t cudaFreeHost(void *p) { free(p); return cudaSuccess; }
 cudaError_t cudaMemPoolCreate(cudaMemPool_t *p, const struct cudaMemPoolProps *q) {
   (void)q;

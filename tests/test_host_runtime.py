@@ -30,8 +30,8 @@ def runtime(tmp_path_factory):
     h4d.lib()  # built before the children load it
     out = tmp_path_factory.mktemp("host") / "fake_cudart.so"
     inc = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
-    subprocess.check_call(["gcc", "-O1", "-Wall", "-fPIC", "-shared", "-I", inc, "-o", str(out),
-                           os.path.join(ROOT, "tests", "host", "fake_cudart.c")])
+    subprocess.check_call(["gcc", "-O1", "-Wall", "-fexceptions", "-fPIC", "-shared", "-I", inc, "-o", str(out),
+                           os.path.join(ROOT, "tests", "host", "fake_cudart.c"), "-lstdc++"])
 
     def run(code):
         env = dict(os.environ, LD_PRELOAD=str(out), PYTHONPATH=ROOT)
@@ -105,5 +105,39 @@ for _ in range(2):
     rt.cudaDeviceReset()
     grad()
     grad()
+print("ok")
+""")
+
+
+def test_no_exception_crosses_the_interface(runtime):
+    runtime("""
+L, p = cfg["L"], h4d.make_params(cfg)
+x = np.random.default_rng(1).uniform(0, L, (100, 3))
+w, f, t = np.zeros(h4d.H4D_PROP_NW), np.zeros((64, 2, 96), np.float32), np.zeros((64, 2), np.float32)
+ctx, _ = context(2)
+rt.fake_device_bytes.restype = ctypes.c_size_t
+
+def out_of_memory(call, at_least):
+    held, failed = rt.fake_device_bytes(), 0
+    for k in range(60):
+        rt.fake_fail_new(k)
+        try:
+            call()
+        except h4d.H4DError as e:
+            failed += 1
+            assert e.code == h4d.H4D_ECUDA, e
+            assert rt.fake_device_bytes() <= held, k  # (a failed context gives the pool back too)
+        finally:
+            rt.fake_fail_new(-1)
+    assert failed >= at_least, failed
+
+out_of_memory(lambda: h4d.h4d_proposal_grad(w, f, t), 1)  # first, while it makes the scratch pool
+out_of_memory(lambda: h4d.h4d_eval_forces(p, L, x), 2)
+out_of_memory(lambda: h4d.h4d_eval_forces_static(p, L, x), 1)
+out_of_memory(lambda: context(2)[0].close(), 5)
+rt.fake_fail_pinned(1)
+ctx, _ = context(2)  # one without a pinned buffer yet
+out_of_memory(lambda: ctx.h4d_get_state(0), 1)
+out_of_memory(lambda: ctx.h4d_get_work(0, 4), 1)
 print("ok")
 """)
