@@ -3214,7 +3214,7 @@ __global__ void __launch_bounds__(512) point_kernel(const __grid_constant__ Poin
         fy = sy;
         fz = sz;
         if (q == 0) {
-          const int tk = ti * 4 + tj;
+          const int t64 = type_of(i, a.nw3), tk = t64 * 4 + type_of(j, a.nw3);  // (type_t ignores waters of LJ systems)
           const u64 d2 = fixed_d2(pi, pj);
           double r264 = r2_of(d2, S);
           double kqg = P.dkq[tk];
@@ -3227,7 +3227,7 @@ __global__ void __launch_bounds__(512) point_kernel(const __grid_constant__ Poin
             if (screened) kqg *= gscr64;
           }
           const double y = P.etab_n > 0 ? pair_add64(P, a.etab, tk, r264, kqg, lj, co, -comp)
-                                        : pair_u64(P, ti, tj, r264, screened ? gscr64 : 1.0) - comp;
+                                        : pair_u64(P, t64, tk - 4 * t64, r264, screened ? gscr64 : 1.0) - comp;
           const double t = part + y;  // Kahan's sum over the lane's pairs
           comp = (t - part) - y;
           part = t;

@@ -90,3 +90,14 @@ def test_rows_near_their_capacity_go_through_the_lists(n_ball):
     Ug, Fg = h4d.h4d_eval_forces(p, L, x)
     assert np.all(np.linalg.norm(Fg - Fo, axis=1) <= force_bounds(cfg, x, Fo))
     assert abs(Ug - Uo) <= 1e-13 * (abs(Uo) + 140)
+
+
+@pytest.mark.parametrize("alpha", [0.3, 0.9])  # Coulomb table, library erfc
+def test_waters_in_an_lj_system_have_the_energy_of_their_types(alpha):
+    cfg = wl.lj_config(250, 0.2, 10, alpha=alpha)
+    x = quantize(wl.lj_positions(125, cfg["L"], 7), cfg["L"])
+    p = h4d.make_params(cfg)
+    Up, _ = h4d.h4d_eval_forces(p, cfg["L"], x, n_water=8)
+    Ue, _ = h4d.h4d_eval_forces_static(p, cfg["L"], x, n_water=8)
+    assert Up == pytest.approx(Ue, rel=1e-12)
+    assert Up != pytest.approx(h4d.h4d_eval_forces(p, cfg["L"], x)[0], rel=1e-6)
