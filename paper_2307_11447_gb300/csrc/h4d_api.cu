@@ -1004,8 +1004,9 @@ static int make_plan(h4d_ctx* c, const std::vector<double>* weight = nullptr) {
     W += w[r];
   }
   size_t max_smem = 0;
-  int min_atoms = 1 << 30, max_atoms = 0;
+  int min_atoms = 1 << 30, max_atoms = 0, max_now = 0;
   for (int r = 0; r < R; ++r) {
+    max_now = std::max(max_now, c->rep_h[r].nw3 + unit_of(c->prm) * c->rep_h[r].n_pairs);
     max_smem = std::max(max_smem, group_smem_bytes(c->rep_h[r].cap_atoms, c->rep_h[r].nc, 0));
     min_atoms = std::min(min_atoms, c->rep_h[r].cap_atoms);
     max_atoms = std::max(max_atoms, c->rep_h[r].cap_atoms);
@@ -1015,10 +1016,14 @@ static int make_plan(h4d_ctx* c, const std::vector<double>* weight = nullptr) {
   // so the launch no longer waits on them alone.  Equal replicas keep two 16-warp CTAs.
   const bool uneven = max_atoms > 2 * min_atoms;
   // A launch of no more replicas than SMs also gives each 32 warps, as half of each SM's warps
-  // would idle otherwise: 64 chains of 4000 ions 295 -> 225 us per MD step, 16 of 1000 ions 73
-  // -> 61 us.  A lone replica keeps 16: its plan is part of what callers check, and at 250 ions
-  // the time is the same.
-  const bool one_per_sm = max_smem > kCtaSmem || uneven || (R > 1 && R <= c->sm_count);
+  // would idle otherwise, from 300 atoms on: smaller ones have too few rows for them and lose more
+  // at the wider barriers.  MD step / trial of 50 steps with 16 and 32 warps, 152 chains: 100 ions
+  // 11.4 and 14.5 / 652 and 768 us, 250 ions (density 0.2) 20.0 and 21.6 / 1246 and 1308, 300 ions (0.45)
+  // 32.9 and 34.4 / 2310 and 2316 (with the learned proposal 5% less with 32), 400 ions (0.3) 34.5
+  // and 33.2 / 2233 and 2084, 1000 ions 76.6 and 64.5 / 5139 and 4281, 4000 ions 313 and 222 / 21591 and
+  // 16259.  A lone replica keeps 16 warps, as before this rule (32 would take 1000 ions from 68.7 to
+  // 59.9 us per step).
+  const bool one_per_sm = max_smem > kCtaSmem || uneven || (R > 1 && R <= c->sm_count && max_now >= 300);
   const int cta_warps = one_per_sm ? kMaxCtaWarps : kCtaWarps;
   const size_t cta_smem = one_per_sm ? (size_t)227 * 1024 : kCtaSmem;
   const int max_ctas = c->sm_count * (one_per_sm ? 1 : 2);  // one resident wave
