@@ -31,7 +31,7 @@
  *     All other device memory is owned by the context and freed by h4d_destroy(), except
  *     for scratch of the stateless calls: up to 16 MiB of it per device stay with the library
  *     between calls (after calls of several threads, up to what they used at once, until the
- *     next wait on the device); h4d_destroy() of any context gives it back.
+ *     next wait on the device); h4d_destroy() gives back what is kept on the current device.
  *   - Each context issues its work on the CUDA stream given at creation; with NULL the
  *     context creates a non-blocking stream of its own (CUDA-graph capture cannot use
  *     the legacy default stream) and destroys it in h4d_destroy().  Launching entry
@@ -102,7 +102,10 @@ typedef struct h4d_params {
                              a Verlet refresh rebuilds both lists once the two largest
                              displacements since the outer build exceed skin_outer - skin */
   int32_t max_nbr;        /* neighbour-row capacity per atom; 0 = derived from density */
-  int32_t threads_per_atom; /* 1,2,4,8,16 or 32; 0 = chosen per replica size (h4d_autotune measures) */
+  int32_t threads_per_atom; /* 1,2,4,8,16 or 32: parts that a neighbour row is dealt to, one lane each;
+                               0 = chosen per replica size (h4d_autotune measures), where a lane of
+                               an LJ system may take several parts: the parts fix the order of a
+                               row's sum and so the bits of the results, the lanes do not */
   int32_t exchange;       /* H4D_EXCHANGE_PAIR, or H4D_EXCHANGE_SINGLE: LJ system only, charges 0,
                              every ion-block atom is one species with the parameters of
                              type 0, and the "pair" counts of h4d_system, h4d_counts and the
@@ -152,7 +155,7 @@ typedef struct h4d_counts {
   double t_build_ns;        /* of which: neighbour-list builds */
   double t_force_ns;        /* of which: FP32 force passes */
   double t_energy_ns;       /* of which: FP64 end-point energies */
-  int64_t threads_per_atom; /* lanes that share one neighbour row in the force pass */
+  int64_t threads_per_atom; /* parts of a neighbour row in the force pass (see h4d_params) */
   int64_t nbr_refreshes;    /* Verlet-row refreshes filtered from the outer rows (between builds) */
   double t_filter_ns;       /* part of t_build_ns spent filtering Verlet rows from outer rows */
   int64_t last_smid;        /* SM that ran this replica's warps in the most recent launch */
@@ -187,7 +190,7 @@ typedef struct h4d_record {
 /* ---- context lifetime ---- */
 
 /* Create a context: copies params and the initial replicas to the device, sizes every
- * buffer for cap_pairs, picks the lanes per neighbour row by replica size when
+ * buffer for cap_pairs, picks the parts per neighbour row and their lanes by replica size when
  * threads_per_atom == 0 (h4d_autotune then measures and keeps the fastest).
  * seed keys the random stream.  cuda_stream is a cudaStream_t (NULL = a stream the context
  * creates and owns). */
@@ -254,7 +257,9 @@ int h4d_run_trials(h4d_ctx* ctx, int64_t k_cycles, int32_t n_eq);
  * one force pass and of one neighbour build per replica. */
 int h4d_autotune(h4d_ctx* ctx, int32_t n_iter, double* host_pass_ns, double* host_build_ns);
 
-/* ---- getters (synchronise the context stream) ---- */
+/* ---- getters (synchronise the context stream) ----
+ * h4d_get_counts, h4d_get_work and h4d_get_state may be called from several threads at once and
+ * with any current device. */
 int h4d_get_counts(h4d_ctx* ctx, int32_t replica, h4d_counts* out);
 /* current FP64 potential and kinetic energy of a replica */
 int h4d_get_energies(h4d_ctx* ctx, int32_t replica, double* U, double* K);
@@ -365,14 +370,14 @@ int h4d_proposal_grad(const double* host_w, int64_t n_rec, const float* host_fea
                       double* loss, double* host_grad);
 
 /* ---- checkpoint ----
- * h4d_save writes a flat binary image (magic "HH4D0004", seed, replica table, positions,
+ * h4d_save writes a flat binary image (magic "HH4D0005", seed, replica table, positions,
  * velocities, trial records) of a context; it synchronises.  h4d_load restores it into a
  * context created with the same system (replica count, atom capacities, waters, box edges
  * and ion capacities must match, else H4D_EINVAL and nothing is changed): each chain's
  * ion count, counters, random-number keys and counters, statistics and records come from the file,
  * the context keeps its own geometry, thresholds, launch plan, proposal grid and record
- * rings.  Out-of-range fields (ion count above capacity, negative record count, an
- * lane count that is not a power of two up to 32) are rejected.  A resumed chain continues bit-identically. */
+ * rings.  Out-of-range fields (ion count above capacity, negative record count, a
+ * part count that is not a power of two up to 32) are rejected.  A resumed chain continues bit-identically. */
 int h4d_save(h4d_ctx* ctx, const char* path);
 int h4d_load(h4d_ctx* ctx, const char* path);
 
@@ -411,12 +416,14 @@ int h4d_eval_forces_static(const h4d_params* params, double L, int32_t n_water, 
  *   U_recip = g (2 pi K / V) sum_{k != 0} exp(-k^2 / 4 alpha^2) / k^2 |S(k)|^2,
  *   S(k) = sum_j q_j exp(i k.r_j), k = 2 pi n / L over 0 < max_d |n_d| <= kmax;
  *   U_self = -g K alpha / sqrt(pi) sum_j q_j^2;
- *   host_F (may be NULL) [n][3] = -dU_recip/dx (FP32 sums of k-vector tiles, FP64 totals).
+ *   host_F (may be NULL) [n][3] = -dU_recip/dx (FP32 sums over at most 512 atoms or products,
+ *   FP64 totals).
  * Charges follow the atom layout of h4d_eval_forces (params->q by type, K = params->kcoul);
  * host_x [n][3] in [0, L) (wrapped otherwise).  Intramolecular exclusion corrections of
  * rigid waters are not included (they do not depend on the positions of other molecules).
- * t_kernel_ms (may be NULL) receives the device time of the two kernels (structure factors,
- * forces), from CUDA events recorded around each launch.
+ * t_kernel_ms (may be NULL) receives the device time of the kernels (grid positions, structure
+ * factors, their sums, forces, their sums), from CUDA events recorded before the first and after
+ * the last.
  * H4D_EINVAL for alpha <= 0, kmax outside 1..64, negative wbar or kappa_lr.  Allocates
  * device scratch per call; runs on the legacy default stream and synchronises it. */
 int h4d_ewald_lr(const h4d_params* params, double L, int32_t n_water, int32_t n, const double* host_x,

@@ -243,8 +243,8 @@ __device__ __forceinline__ void pair_fr_lj2_poly(const Pot& P, float2 r2, float2
 }
 
 // Two aqueous pair terms at once: the operations of pair_fr<H4D_SYS_AQ> in the same order, each
-// half rounded like its scalar counterpart.  t: sigma^2, 4 epsilon and charge product of each
-// pair; kqg: the charge products times their screening factors.  FIT: erfc from the fitted erfcx.
+// half rounded like its scalar counterpart.  sig2, eps4: sigma^2 and 4 epsilon of each pair; kqg: the
+// charge products times their screening factors.  FIT: erfc from the fitted erfcx.
 template <bool FIT>
 __device__ __forceinline__ float2 pair_fr_aq2(const Pot& P, float2 r2, float2 sig2, float2 eps4, float2 kqg) {
   const float2 rinv = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
@@ -419,11 +419,12 @@ struct Ctx {
   __device__ void sync() const { gsync(bar, T); }
 };
 
-// Row slot s of atom i lives in packet P = s/4 (element s%4).  Packets are dealt to the
-// atom's tpa lanes round-robin (lane P % tpa, its (P / tpa)-th packet), and the packets of
-// consecutive atoms are adjacent, so one 8-byte load per lane gives four neighbours and a
-// warp reads 256 contiguous bytes.  Builders fill a row packet by packet and store whole
-// packets; the last packet of a row is padded with kNoAtom.
+// Verlet rows: slot s of the row at position k lives in packet P = s/4 (element s%4).  Packets are
+// dealt to tpa parts round-robin (part P % tpa, its (P / tpa)-th packet), and the packets of
+// consecutive positions are adjacent, so one 8-byte load gives four neighbours and a warp reads
+// 256 contiguous bytes.  The filter stores whole packets, the last one padded with the sentinel's
+// index (outer rows are not padded: what lies beyond their count is not read).  kNoAtom marks the
+// empty slots of the cell-sorted list.
 constexpr uint16_t kNoAtom = 0xFFFF;
 __device__ __forceinline__ size_t packet_index(const Eng& e, const RepC& R, int i, int P, int ltpa) {
   return (size_t)R.atom_off * e.max_nbr / 4 + ((((size_t)(P >> ltpa) * R.cap_atoms + i) << ltpa) + (P & ((1 << ltpa) - 1)));
@@ -542,10 +543,6 @@ __device__ __forceinline__ u64 fixed_d2(const uint4& a, const uint4& b) {
 __device__ __forceinline__ unsigned d2_16(const uint4& a, const uint4& b) {
   const int dx = (int)(a.x - b.x) >> 16, dy = (int)(a.y - b.y) >> 16, dz = (int)(a.z - b.z) >> 16;
   return (unsigned)(dx * dx) + (unsigned)(dy * dy) + (unsigned)(dz * dz);
-}
-
-__device__ __forceinline__ bool excluded_pair(int i, int j, int nw3) {
-  return i < nw3 && j < nw3 && (i / 3) == (j / 3);
 }
 
 // Verlet-row layout by row length (see next_rank): 64 length buckets; replicas of fewer
@@ -720,7 +717,7 @@ __device__ __forceinline__ int outer_rows(const Ctx& c, int n, bool use_rank) {
 // order.  A warp takes four home atoms, one candidate per lane, and a ballot compacts the
 // accepted ones (about half of them), whose lanes store their indices.  These systems are small,
 // so latency decides: 250 atoms are 63 items for the group's warps, where 32 homes per warp
-// (outer_rows) made 8 items of four times the length.  Outer build of one 250-ion chain: 38 ->
+// (outer_rows) made 8 items of four times the length.  Outer build of one 250-ion chain: 33 ->
 // 22 us.
 template <bool WATER>
 __device__ __forceinline__ int outer_rows_all(const Ctx& c, int n, bool use_rank) {
@@ -984,8 +981,9 @@ __device__ H4D_PHASE void filter_list_impl(const Ctx& cref) {
 // gathers 57%, ALU 36% busy).  With the LJ cut-off inside, a pair beyond it skips the addition
 // of the LJ term and one beyond both skips the three force sums, all predicated; selecting
 // zeros instead took four instructions more per pair, and rsqrtf's rescaling of subnormal
-// arguments three.  The results are the same bits: adding a zero term changes no sum.  Force
-// passes of 304 chains of 4000 ions inside the engine: 218 -> 207 us.
+// arguments three.  The results are the same bits: adding a zero term changes no sum.  MD steps
+// of 304 chains of 4000 ions 437 -> 425 us (when written; a force pass on one lane per row now takes
+// 180 us inside the engine, 157 us alone).
 template <bool NEMD, int FORM>
 __device__ __forceinline__ void lj_row(const Pot& P, const uint4* __restrict__ pos, const uint2* pk, size_t pstride,
                                        int npk, uint2 q, int i, const uint4& pi, float scale, float wi,
@@ -1104,7 +1102,8 @@ __device__ __forceinline__ void aq_row(const Pot& P, const uint4* __restrict__ p
 }
 
 // ------------------------------------------------------------------------------------
-// Force pass (FP32): tpa lanes per atom over its full row, butterfly reduction.
+// Force pass (FP32): the tpa parts of an atom's full row on tpa lanes, or on fewer that take several
+// parts each; butterfly reduction.
 // mode bits: 1 = apply the second half kick, 2 = accumulate kinetic partials,
 //            4 = flyer rows compute protocol work with previous altitude w_prev
 // ------------------------------------------------------------------------------------
@@ -3130,7 +3129,7 @@ int launch_eval(const Eng& e, int threads, size_t smem, float wbar, double* U, v
 // ------------------------------------------------------------------------------------
 // Single-point forces and energy of one configuration over the whole GPU
 // ------------------------------------------------------------------------------------
-// A warp per home atom (kHomes of them in turn): it runs over all atoms, 32 per step, with the
+// A warp per home atom (a.homes of them in turn): it runs over all atoms, 32 per step, with the
 // exact integer distance test, and queues the ones inside the cut-off in shared memory, pairs
 // whose energy this atom owns apart from the others; a full queue of 32 is one FP32 force term
 // per lane and, for the owned pairs, one FP64 energy term, so no lane of the slow FP64 pipe
@@ -3139,7 +3138,7 @@ int launch_eval(const Eng& e, int threads, size_t smem, float wbar, double* U, v
 // 9110 atoms).  The lists' capacities are still part of the call: two counts per home bound the
 // rows that the list build would make, and the host takes that path when a row could overflow.
 // Calls of h4d_eval_forces: 2.9 ms for 1000 ions and 13.9 ms for 400 waters with the engine's lists
-// on one CTA, 0.30 and 0.26 ms with this kernel.
+// on one CTA, 0.145 and 0.097 ms with this kernel, the scratch pool and the table's series kept.
 struct TwoF {  // unevaluated sum
   float hi, lo;
 };
@@ -3278,8 +3277,10 @@ __global__ void __launch_bounds__(512) point_kernel(const __grid_constant__ Poin
   if (lane == 0) a.u_part[blockIdx.x * nwarps + warp] = part;
 }
 
-// warps per CTA and homes per warp: about one wave of 16 warps per SM, with 8-warp CTAs while
-// those alone do not cover the SMs twice (1000 ions: 125 CTAs instead of 63)
+// warps per CTA and homes per warp: one home per warp and 8-warp CTAs up to 16 warps per SM (1000
+// ions: 125 CTAs instead of 63 of 16 warps, 2432 atoms: 304), then 16-warp CTAs and the homes that
+// keep them to one wave.  From 2433 atoms on the second home halves the CTAs to 77, so up to about
+// 4800 atoms part of the SMs idle.
 int point_plan(int n, int* warps, int* homes, int* ctas) {
   *homes = (n + 152 * 16 - 1) / (152 * 16);
   *warps = n <= 152 * 16 ? 8 : 16;

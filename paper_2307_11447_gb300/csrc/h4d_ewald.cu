@@ -57,7 +57,7 @@ __device__ __forceinline__ int2 column(int c, int kmax) {
 
 // cos and sin of 2 pi ph / 2^32: the nearest quarter turn is taken off in integers, and on the
 // remaining eighth of a turn either side the Taylor polynomials (first omitted terms: 2e-9 of
-// the sine, 1.1e-9 of the cosine) need no further reduction.  Half the instructions of
+// the sine, 1.2e-10 of the cosine) need no further reduction.  Half the instructions of
 // sincospif on the converted phase, whose conversion also rounds a whole turn to 24 bits.
 __device__ __forceinline__ void phase_cs(unsigned ph, float& c, float& s) {
   const unsigned k = ph + 0x20000000u;  // its top two bits: the quarter turn
