@@ -399,9 +399,8 @@ int h4d_eval_forces(const h4d_params* params, double L, int32_t n_water, int32_t
  * gives *U = 0 and touches no device memory).  It
  * calls no cudaMalloc, cudaFree or other allocating routine: every device buffer lives in
  * one file-scope array of 16 MiB that each GPU loading the library holds until the
- * process exits.  The first call on a device looks up that array's device address
- * (cudaGetSymbolAddress) with the device current; make that first call before any stream
- * capture.  Sizes that do not fit (about 6000 LJ atoms with default capacities) return
+ * process exits.  Each call looks up that array's device address (cudaGetSymbolAddress) in the
+ * current context; make the first call on a device before any stream capture.  Sizes that do not fit (about 6000 LJ atoms with default capacities) return
  * H4D_ECAPACITY.  All calls share the array and it keeps the last call's contents (each
  * call writes everything it reads); calls that overlap on the GPU -- from several host
  * threads or processes sharing a context -- race on it and must be serialised by the

@@ -1846,22 +1846,11 @@ int h4d_neighbor_pairs(double L, int32_t n, const double* x, double r_list, int3
 static constexpr size_t kStaticScratchBytes = 16u << 20;  // 16 MiB
 static __device__ __align__(256) unsigned char g_h4d_static_scratch[kStaticScratchBytes];
 
-// The array's name in host code is only a host-side stand-in: its device address comes
-// from cudaGetSymbolAddress, once per device, with that device current.
-static std::mutex g_static_mu;
-static void* g_static_addr[64];
-
+// The array's name in host code is only a host-side stand-in: its device address comes from
+// cudaGetSymbolAddress, on every call, as it belongs to the current context (another device, or the
+// same one after cudaDeviceReset, has another).
 static int static_scratch_address(void** out) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return H4D_ECUDA;
-  std::lock_guard<std::mutex> lock(g_static_mu);
-  if (!g_static_addr[dev]) {
-    void* p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_h4d_static_scratch) != cudaSuccess || !p) return H4D_ECUDA;
-    g_static_addr[dev] = p;
-  }
-  *out = g_static_addr[dev];
-  return H4D_OK;
+  return cudaGetSymbolAddress(out, g_h4d_static_scratch) == cudaSuccess && *out ? H4D_OK : H4D_ECUDA;
 }
 
 // doubles in, fixed-point box fractions out (same rule as to_fixed: wrap into [0, L),

@@ -5,13 +5,14 @@
  * current one is refused, as CUDA does.  A memory pool keeps what is freed to it until the
  * next wait and then, if that is more than its release threshold, gives it back;
  * fake_device_bytes() is what the devices hold.  cudaDeviceReset ends the context: a pool
- * made before it is refused.  fake_fail_new(k) makes this thread's k-th C++ allocation from then on
+ * made before it is refused, device variables move and their old memory is gone.  fake_fail_new(k) makes this thread's k-th C++ allocation from then on
  * throw (-1: none), fake_fail_pinned(1) every allocation of pinned memory fail. */
 #include <cuda.h>
 #include <cuda_runtime_api.h>
 #include <stdint.h>
 #include <stdlib.h>
 #include <string.h>
+#include <sys/mman.h>
 #include <unistd.h>
 
 static __thread int t_dev;
@@ -28,6 +29,7 @@ static cudaError_t ret(cudaError_t e) {
 static size_t held;
 struct pool { size_t idle; unsigned long long keep; int dead; };
 static unsigned long long ctx_id = 1;
+static void *symbol;  /* the library's device variable */
 struct head { size_t n; struct pool *from; char fill[240]; };
 static struct pool *pools[16];
 static int n_pools;
@@ -117,6 +119,7 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void **a, size_t 
 }
 
 /* ---- devices, streams, memory ---- */
+cudaError_t cudaGetSymbolAddress(void **p, const void *s);
 static CUresult ctx_get_id(CUcontext c, unsigned long long *id) { (void)c; *id = ctx_id; return CUDA_SUCCESS; }
 cudaError_t cudaGetDriverEntryPointByVersion(const char *name, void **f, unsigned v, unsigned long long fl,
                                              enum cudaDriverEntryPointQueryResult *st) {
@@ -127,6 +130,11 @@ cudaError_t cudaGetDriverEntryPointByVersion(const char *name, void **f, unsigne
 }
 cudaError_t cudaDeviceReset(void) {
   for (int i = 0; i < n_pools; ++i) { trim(pools[i], 0); pools[i]->dead = 1; }
+  if (symbol) {
+    void *old = symbol;
+    cudaGetSymbolAddress((symbol = 0, &symbol), 0); /* at another address */
+    munmap(old, 16 << 20);
+  }
   ++ctx_id;
   return cudaSuccess;
 }
@@ -166,8 +174,8 @@ cudaError_t cudaMallocHost(void **p, size_t n) {
 }
 cudaError_t cudaGetSymbolAddress(void **p, const void *s) {
   (void)s;
-  static char array[16 << 20];
-  *p = array;
+  if (!symbol) symbol = mmap(0, 16 << 20, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS, -1, 0);
+  *p = symbol;
   return cudaSuccess;
 }
 cudaError_t cudaFreeHost(void *p) { free(p); return cudaSuccess; }

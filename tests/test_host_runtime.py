@@ -109,6 +109,16 @@ print("ok")
 """)
 
 
+def test_static_scratch_is_found_again_after_a_device_reset(runtime):
+    runtime("""
+x = np.random.default_rng(1).uniform(0, cfg["L"], (100, 3))
+for _ in range(3):
+    h4d.h4d_eval_forces_static(h4d.make_params(cfg), cfg["L"], x)
+    rt.cudaDeviceReset()
+print("ok")
+""")
+
+
 def test_no_exception_crosses_the_interface(runtime):
     runtime("""
 L, p = cfg["L"], h4d.make_params(cfg)
